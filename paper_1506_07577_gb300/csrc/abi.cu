@@ -148,6 +148,8 @@ void free_tet_data(ebb_rel_s* r) {
   free_edges(r);
   free_layout(r);
   free_step_scratch(r);
+  free_row_step(r);
+  free_row_matrix(r);
   free_batch_scratch(r);
   r->finalized = false;
 }

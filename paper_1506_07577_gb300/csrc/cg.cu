@@ -878,9 +878,18 @@ ebb_status_t run_implicit_step(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, doubl
     if (rep) rep->status = EBB_OK;
     return EBB_OK;
   }
+  const bool f64 = p->precision == EBB_PREC_F64;
+  // FP64 steps run on the assembled rows (row_step.cu) where those apply.  A
+  // caller that asks for the edge relation's blocks (EBB_STEP_ASSEMBLED) gets
+  // them below, where the step leaves them assembled for ebb_spmv_tet_K.
+  if (f64 && !(p->flags & EBB_STEP_ASSEMBLED)) {
+    bool rows = false;
+    const ebb_status_t rs = row_step_ready(ctx, tets, &rows);
+    if (rs) return rs;
+    if (rows) return run_row_step(ctx, tets, u, v, pinned, pinned_dtype, p, rep);
+  }
   ebb_status_t s = ensure_scratch(ctx, tets);
   if (s) return s;
-  const bool f64 = p->precision == EBB_PREC_F64;
   if (tets->vperm) {
     // Reordered vertices: the step runs on the state in the internal order.
     StepScratch* sc = tets->step;
@@ -923,6 +932,13 @@ ebb_status_t run_step_vjp(ebb_ctx_s* ctx, ebb_rel_s* tets, const double* u, cons
   if (tets->verts->size == 0) {
     if (rep) rep->status = EBB_OK;
     return EBB_OK;
+  }
+  {
+    bool rows = false;
+    const ebb_status_t rs = row_step_ready(ctx, tets, &rows);
+    if (rs) return rs;
+    if (rows)
+      return run_row_vjp(ctx, tets, u, v, v_next, pinned, pinned_dtype, gu, gv, gmu, glam, p, rep);
   }
   ebb_status_t s = ensure_scratch(ctx, tets);
   if (s) return s;

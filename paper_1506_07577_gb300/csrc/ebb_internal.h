@@ -192,6 +192,8 @@ inline int chunk_first_tile(int c, int ntiles, int K) {
 }
 
 struct BatchScratch;  // defined in batched.cu
+struct RowMatrix;     // defined in row_matrix.cuh
+struct RowStep;       // defined in row_step.cu
 
 struct ebb_rel_impl;
 
@@ -238,6 +240,8 @@ struct ebb_rel_s {
 
   // ---- implicit-step scratch ----
   ebb::StepScratch* step = nullptr;
+  ebb::RowMatrix* rows = nullptr;       // row matrix pattern (row_matrix.cu), built on first use
+  ebb::RowStep* row_step = nullptr;     // FP64 step on the rows (row_step.cu)
   ebb::HostPlan* hplan = nullptr;       // chunk plan of the host-buffer map (abi.cu)
   float* xyz_stage = nullptr;           // host-buffer map's packed-row staging: u, w, f, Kw, 3 x N_v floats
                                         // each (EBB_MAP_HOST_XYZ; allocated on first use)
@@ -334,6 +338,18 @@ ebb_status_t rebuild_tiles(ebb_ctx_s* ctx, ebb_rel_s* tets, int cap);
 // Rewrite the per-tet part of every blob in the record layout `planes`
 // (the tiles stay as they are).
 ebb_status_t repack_records(ebb_ctx_s* ctx, ebb_rel_s* tets, bool planes);
+
+// FP64 step and step VJP on the assembled row matrix (row_step.cu).
+// row_step_ready builds what they need on first use and says whether they
+// apply to the relation; the other calls follow a *yes.
+ebb_status_t row_step_ready(ebb_ctx_s* ctx, ebb_rel_s* tets, bool* yes);
+ebb_status_t run_row_step(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, const void* pinned,
+                          ebb_dtype_t pinned_dtype, const ebb_step_params_t* p, ebb_cg_report_t* rep);
+ebb_status_t run_row_vjp(ebb_ctx_s* ctx, ebb_rel_s* tets, const double* u, const double* v, const double* v_next,
+                         const void* pinned, ebb_dtype_t pinned_dtype, double* gu, double* gv, double* gmu,
+                         double* glam, const ebb_step_params_t* p, ebb_cg_report_t* rep);
+void free_row_step(ebb_rel_s* tets);
+void free_row_matrix(ebb_rel_s* tets);
 
 // Step VJP (cg.cu) and its adjoint element map (adjoint.cu).
 // v_next (may be null): the step's new velocity, which replaces its forward

@@ -1,0 +1,71 @@
+// Row matrix of a tets relation: the assembled stiffness with three lanes per
+// vertex row (device layout, shared by the assembly, the product and the CG
+// solve on it).
+//
+// A vertex's row holds one 3x3 block per vertex that shares a tet with it,
+// itself first (slot 0), the others by increasing vertex number.  Rows are
+// gathered into slices of kSliceRows rows; lane 3 i + c of a warp owns
+// component c of the slice's row i (30 of 32 lanes).  A slice has as many
+// slots as its longest row.  Slot k of slice s is slot number
+// slice_off[s] + k =: q, and holds
+//   col[q * kSliceRows + i]        vertex of row i's k-th block
+//   val[(q * 3 + d) * 32 + lane]   the block's entry (c, d)
+// so that every load of a warp is one line of consecutive words, and a
+// lane's product is a plain sum over its own entries, with no reduction
+// between lanes: on GB300 an FP64 add costs a warp 64 cycles, so adds that
+// only combine lanes are what the layout avoids.  Unused entries are zero and
+// unused columns name the row's own vertex.
+//
+// Rows enter the slices in windows of kWindowRows vertices (taken in order of
+// first use by the tets, so that neighbours stay close), sorted by length
+// within the window: a slice's rows then have nearly equal lengths, whatever
+// the vertex numbering.
+#pragma once
+
+#include <cstdint>
+
+#include "ebb_internal.h"
+
+namespace ebb {
+
+constexpr int kSliceRows = 10;                       // rows per slice (30 lanes)
+constexpr int kWindowSlices = 32;
+constexpr int kWindowRows = kSliceRows * kWindowSlices;
+constexpr int kRowMaxTets = 128;                     // tets around one vertex
+// Element record, in values: the blocks of the six corner pairs (a < b,
+// pair order 01 02 03 12 13 23, 9 entries each, row-major), then the corner
+// forces of corners 1..3 (corner 0 is minus their sum), one value unused.
+constexpr int kElemLen = 64;
+constexpr int kElemForce = 54;
+
+struct RowMatrix {
+  int state = 0;              // 0 not built, 1 built, -1 does not apply to this relation
+  int nslice = 0;
+  int64_t nslots = 0;
+  int* slice_off = nullptr;   // nslice + 1
+  int* row_of = nullptr;      // nslice * kSliceRows: vertex of each row, -1 for none
+  int* col = nullptr;         // nslots * kSliceRows
+  int2* crange = nullptr;     // nslots * kSliceRows: the block's contributions [x, y)
+  int* slot_slice = nullptr;  // nslots: slice of each slot
+  int* contrib = nullptr;     // 12 per tet, row by row: 16 t + 2 pair + transposed
+};
+
+// The vertex order and index arrays of the matrix, as the kernels take them.
+struct RowView {
+  int nslice;
+  const int* __restrict__ slice_off;
+  const int* __restrict__ row_of;
+  const int* __restrict__ col;
+};
+
+// Build the pattern on first use (device work on `stream`, synchronous).
+// EBB_OK with rm.state == -1: a vertex has more than kRowMaxTets tets, or the
+// memory does not suffice; the caller then keeps to the matrix-free maps.
+ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t stream);
+// Element records of K(u) and, with `force`, the element forces: u in planes
+// (stride nv) or interleaved 4-float elements (aos).
+template <typename T>
+cudaError_t launch_element_blocks(ebb_rel_s* rel, int model, T mu0, T lam0, const T* u, bool aos, bool force, T* elem,
+                                  cudaStream_t st);
+
+}  // namespace ebb
