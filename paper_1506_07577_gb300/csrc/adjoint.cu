@@ -71,32 +71,42 @@ adjoint_stvk_kernel(int nt, int nv, const int4* __restrict__ keys, const int* __
   double F[9];
 #pragma unroll
   for (int i = 0; i < 9; ++i) F[i] = G[i] + ((i % 4) == 0 ? 1.0 : 0.0);
-  // K lam: dP(F; L)
-  double dPl[9];
-  stvk_dP(sv, mu, lam, L, dPl);
   // Q = d/dF [dP(F; W) : L]
-  double FtW[9], WtL[9], FtL[9], sWtL[9], sFtL[9], C[9];
+  double FtW[9], WtL[9], FtL[9], sWtL[9], sFtL[9], sFtW[9], C[9];
   mtm(F, W, FtW);
   mtm(W, L, WtL);
   mtm(F, L, FtL);
   sym3(WtL, sWtL);
   sym3(FtL, sFtL);
-  sym3(FtW, C);
+  sym3(FtW, sFtW);
   const double trFtW = FtW[0] + FtW[4] + FtW[8];
   const double trWtL = WtL[0] + WtL[4] + WtL[8];
   const double trFtL = FtL[0] + FtL[4] + FtL[8];
+  const double mu2 = 2.0 * mu;
+  // The symmetric tangents of the three pairs, Y(A) = 2 mu sym(A) + lam tr(A) I:
+  // dP(F; L) = L S + F Y(F^T L), Q = F Y(W^T L) + L Y(F^T W) + W Y(F^T L).
 #pragma unroll
-  for (int i = 0; i < 9; ++i) C[i] *= 2.0 * mu;
-  C[0] += lam * trFtW;
-  C[4] += lam * trFtW;
-  C[8] += lam * trFtW;
-  double Q[9], T1[9], T2[9], T3[9];
-  mm(F, sWtL, T1);
+  for (int i = 0; i < 9; ++i) {
+    C[i] = mu2 * sFtW[i];
+    WtL[i] = mu2 * sWtL[i];
+    FtL[i] = mu2 * sFtL[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 9; i += 4) {
+    C[i] += lam * trFtW;
+    WtL[i] += lam * trWtL;
+    FtL[i] += lam * trFtL;
+  }
+  double dPl[9], Q[9], T1[9], T2[9], T3[9];
+  mm(L, sv.S, dPl);
+  mm(F, FtL, T1);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) dPl[i] += T1[i];
+  mm(F, WtL, T1);
   mm(L, C, T2);
-  mm(W, sFtL, T3);
+  mm(W, FtL, T3);
 #pragma unroll
-  for (int i = 0; i < 9; ++i)
-    Q[i] = 2.0 * mu * T1[i] + lam * trWtL * F[i] + T2[i] + 2.0 * mu * T3[i] + lam * trFtL * W[i];
+  for (int i = 0; i < 9; ++i) Q[i] = T1[i] + T2[i] + T3[i];
   // corners
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -123,16 +133,11 @@ adjoint_stvk_kernel(int nt, int nv, const int4* __restrict__ keys, const int* __
 #pragma unroll
       for (int j = 0; j < 3; ++j) E[i * 3 + j] = 0.5 * (G[i * 3 + j] + G[j * 3 + i] + GtG[i * 3 + j]);
     const double trE = E[0] + E[4] + E[8];
-    double FE[9], WE[9], FdE[9], dE[9];
-    mm(F, E, FE);
-    mm(W, E, WE);
-    sym3(FtW, dE);
-    mm(F, dE, FdE);
-    const double FL = ddot9(F, L);
-    const double f_mu = -V * 2.0 * ddot9(FE, L);
-    const double f_lam = -V * trE * FL;
-    const double k_mu = V * 2.0 * (ddot9(WE, L) + ddot9(FdE, L));
-    const double k_lam = V * (trE * ddot9(W, L) + trFtW * FL);
+    // (F E) : L = E : F^T L and so on, E symmetric
+    const double f_mu = -2.0 * V * ddot9(E, sFtL);
+    const double f_lam = -V * trE * trFtL;
+    const double k_mu = 2.0 * V * (ddot9(E, sWtL) + ddot9(sFtW, sFtL));
+    const double k_lam = V * (trE * trWtL + trFtW * trFtL);
     const int o = perm[t];
     if (gmu) gmu[o] += dt * f_mu - dt * dt * k_mu;
     if (glam) glam[o] += dt * f_lam - dt * dt * k_lam;

@@ -85,7 +85,8 @@ row_length_kernel(int nv, const int* __restrict__ off, const int* __restrict__ e
 }
 
 // One block per window: rows sorted by decreasing length (ties in order of
-// first use), row_of, where each vertex went, and the slices' slot counts.
+// first use), the slices they make up in alternating quads, where each vertex
+// went, and the slices' slot counts.
 __global__ void __launch_bounds__(kWindowRows)
 window_kernel(int nv, const int* __restrict__ order, const int* __restrict__ len, int* row_of, int* place,
               int* slots) {
@@ -98,9 +99,13 @@ window_kernel(int nv, const int* __restrict__ order, const int* __restrict__ len
   __syncthreads();
   int rank = 0;
   for (int j = 0; j < kWindowRows; ++j) rank += s_len[j] > l || (s_len[j] == l && j < i);
-  row_of[blockIdx.x * kWindowRows + rank] = v;
-  if (v >= 0) place[v] = blockIdx.x * kWindowRows + rank;
-  if (rank % kSliceRows == 0) slots[blockIdx.x * kWindowSlices + rank / kSliceRows] = l;
+  // slices by decreasing length; quads of them alternate from both ends
+  const int sl = rank / kSliceRows, quad = sl / 4;
+  const int pos = 4 * (quad < kWindowSlices / 8 ? 2 * quad : 2 * (kWindowSlices / 4 - 1 - quad) + 1) + sl % 4;
+  const int at = (blockIdx.x * kWindowSlices + pos) * kSliceRows + rank % kSliceRows;
+  row_of[at] = v;
+  if (v >= 0) place[v] = at;
+  if (rank % kSliceRows == 0) slots[blockIdx.x * kWindowSlices + pos] = l;
 }
 
 // Exclusive sums of n counts into out[0 .. n], by one block.
@@ -415,6 +420,9 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
   if (e == cudaSuccess) e = cudaMalloc(&m->slice_off, ((size_t)m->nslice + 1) * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&m->row_of, (size_t)nwin * kWindowRows * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&m->contrib, std::max<size_t>(1, (size_t)nt * 12) * sizeof(int));
+  int nsm = 0;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device);
+  m->grid = std::min({std::max(nsm, 1), kRowMaxGrid, m->nslice});
   int host[2] = {0, 0};   // total slots, too-long flag
   int *len = tmp, *place = tmp + nv, *slots = tmp + 2 * (size_t)nv, *flag = slots + m->nslice;
   const int sort_grid = (nv + kSortWarps - 1) / kSortWarps;
@@ -457,7 +465,7 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
     cudaFree(m->crange);
     cudaFree(m->slot_slice);
     cudaFree(m->contrib);
-    *m = RowMatrix();
+      *m = RowMatrix();
     m->state = -1;
     if (e == cudaSuccess || e == cudaErrorMemoryAllocation) {
       cudaGetLastError();

@@ -32,6 +32,7 @@ constexpr int kSliceRows = 10;                       // rows per slice (30 lanes
 constexpr int kWindowSlices = 32;
 constexpr int kWindowRows = kSliceRows * kWindowSlices;
 constexpr int kRowMaxTets = 128;                     // tets around one vertex
+constexpr int kRowMaxGrid = 256;                     // thread blocks of a kernel over all slices
 // Element record, in values: the blocks of the six corner pairs (a < b,
 // pair order 01 02 03 12 13 23, 9 entries each, row-major), then the corner
 // forces of corners 1..3 (corner 0 is minus their sum), one value unused.
@@ -48,6 +49,7 @@ struct RowMatrix {
   int2* crange = nullptr;     // nslots * kSliceRows: the block's contributions [x, y)
   int* slot_slice = nullptr;  // nslots: slice of each slot
   int* contrib = nullptr;     // 12 per tet, row by row: 16 t + 2 pair + transposed
+  int grid = 0;               // thread blocks of a kernel over all slices (at most one per SM)
 };
 
 // The vertex order and index arrays of the matrix, as the kernels take them.
@@ -57,6 +59,11 @@ struct RowView {
   const int* __restrict__ row_of;
   const int* __restrict__ col;
 };
+
+// First slice of block b of `grid`, which take consecutive slices.
+__host__ __device__ inline int first_slice(int b, int grid, int nslice) {
+  return (int)((long long)b * nslice / grid);
+}
 
 // Build the pattern on first use (device work on `stream`, synchronous).
 // EBB_OK with rm.state == -1: a vertex has more than kRowMaxTets tets, or the

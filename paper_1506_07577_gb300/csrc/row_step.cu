@@ -14,8 +14,8 @@
 // No atomics on floating-point data: results repeat bit for bit, whatever
 // reduction the caller names.
 // Measured, against the matrix-free step with two launches per iteration: 8^3
-// StVK step (2,560 tets) 498 -> 165 us; 20-step rollout and gradient on the
-// 32^3 mesh (163,840 tets) 213 -> 51 ms.
+// StVK step (2,560 tets) 498 -> 138 us; 20-step rollout and gradient on the
+// 32^3 mesh (163,840 tets) 213 -> 46 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -52,7 +52,7 @@ namespace {
 
 constexpr int kPlainThreads = 768;   // row_cg_kernel, one CTA per SM
 constexpr int kSplitThreads = 128;   // its form for few slices
-constexpr int kMaxGrid = 256;        // partial sums per set
+constexpr int kMaxGrid = kRowMaxGrid;   // partial sums per set
 constexpr long long kGridWaitCycles = 2000000000LL;  // about 1 s at 2 GHz
 
 // Streaming load of a matrix value (read once per product: not kept in L1,
@@ -160,7 +160,8 @@ struct RowCgShared {
   double v[kSums][NP];
   double w[kSums][2];
   double tot[kSums];
-  double scal[4];               // alpha, beta, 1 / r.z, 1 / (r.z alpha)
+  double alpha, beta, pq;       // of this iteration; pq = p.Ap
+  double inv[2];                // 1 / r.z, by iteration parity
   int active, ok;
 };
 
@@ -179,16 +180,17 @@ __device__ __forceinline__ bool wait_acquire(const unsigned* bar, unsigned targe
   }
 }
 
-// Barrier over the grid.  The counter only grows: round r is complete at
+// Barrier over the grid in two halves, so that work no other block waits for
+// can run in between.  The counter only grows: round r is complete at
 // r * gridDim.x arrivals.
-template <int NP>
-__device__ __forceinline__ bool grid_wait(RowCgShared<NP>& sh, unsigned* bar, unsigned& round) {
+__device__ __forceinline__ void grid_arrive(unsigned* bar, unsigned& round) {
   ++round;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    arrive_release(bar);
-    sh.ok = wait_acquire(bar, round * gridDim.x);
-  }
+  if (threadIdx.x == 0) arrive_release(bar);
+}
+template <int NP>
+__device__ __forceinline__ bool grid_join(RowCgShared<NP>& sh, const unsigned* bar, unsigned round) {
+  if (threadIdx.x == 0) sh.ok = wait_acquire(bar, round * gridDim.x);
   __syncthreads();
   return sh.ok != 0;
 }
@@ -255,25 +257,28 @@ __device__ __forceinline__ bool grid_sum(RowCgShared<NP>& sh, const double (&x)[
 //   w = A z;  r.z, w.z, r.r
 //   | beta = r.z / (r.z)', alpha = r.z / (w.z - beta r.z / alpha');  p = z + beta p;
 //     s = w + beta s (= A p);  y += alpha p;  r -= alpha s;  z = r / diag A  |
-// with two grid barriers (|) where the usual form has three; the reduction
-// and the barriers cost as much as the products do (32^3 mesh: 8 us of FP64
-// products and, in the usual form, 15 us of the rest).
+// with two grid barriers (|) where the usual form has three.  Measured on the
+// 32^3 mesh, in SM cycles of an iteration: product 20,000 (17,500 at the FP64
+// issue rate), reduction 8,500 (5,000 when no block is late), scalars 1,800,
+// vectors 1,300, barrier 3,000; in the usual form with vectors in memory and
+// slices of unequal length the iteration took 50,000.
 // A warp owns whole slices, a lane one component of one row, in every pass,
-// so all vectors but z stay with their thread.  SPLIT: four warps share a
-// slice's slots and the first adds their sums; for meshes with at most three
-// slices per SM, where one warp's chain of FP64 operations (64 cycles each)
-// would be the iteration.
+// so all vectors but z stay with their thread: in registers for the warp's
+// first slice (all of them on meshes of up to 36,000 vertices), in memory for
+// the others.  SPLIT: four warps share a slice's slots and the first adds
+// their sums; for meshes with at most three slices per SM, where one warp's
+// chain of FP64 operations (64 cycles each) would be the iteration.
 template <int NT, bool SPLIT, typename PT>
 __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __restrict__ pin) {
   constexpr int NP = SPLIT ? 32 : NT;
   __shared__ RowCgShared<NP> sh;
   __shared__ double s_acc[SPLIT ? 4 : 1][5][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int G = gridDim.x;
   const bool lane_on = lane < 3 * kSliceRows;
   const int i = lane_on ? lane / 3 : 0, c = lane_on ? lane - 3 * i : 0;
-  const int s0 = SPLIT ? (int)blockIdx.x : (int)blockIdx.x + G * warp;
-  const int sstep = SPLIT ? G : G * (NT / 32);
+  const int first = first_slice(blockIdx.x, gridDim.x, a.m.nslice) + (SPLIT ? 0 : warp);
+  const int last = first_slice(blockIdx.x + 1, gridDim.x, a.m.nslice);
+  constexpr int sstep = SPLIT ? 1 : NT / 32;
   const int k0 = SPLIT ? warp : 0;
   constexpr int kstep = SPLIT ? 4 : 1;
   const bool vec = !SPLIT || warp == 0;   // this warp runs the vector passes
@@ -289,11 +294,54 @@ __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __
     }
     return x;
   };
+  // this lane's entry of A z
+  auto product = [&](int q0, int nk) {
+    double acc = 0.0;
+    const int* col = a.m.col + (size_t)q0 * kSliceRows + i;
+    const double* val = a.val + (size_t)q0 * 96 + lane;
+    // groups of U slots; the next group's columns are loaded a group ahead
+    constexpr int U = SPLIT ? 5 : 3;
+    int j[U];
+#pragma unroll
+    for (int g = 0; g < U; ++g) j[g] = k0 + g * kstep < nk ? col[(k0 + g * kstep) * kSliceRows] : 0;
+    for (int k = k0; k < nk; k += U * kstep) {
+      double x[U][3], w[U][3];
+#pragma unroll
+      for (int g = 0; g < U; ++g) {
+        const bool in = k + g * kstep < nk;
+        const double* xv = a.z + 3 * (size_t)j[g];
+        const double* wv = val + (size_t)(in ? k + g * kstep : 0) * 96;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          x[g][d] = xv[d];
+          w[g][d] = ld_stream(wv + 32 * d);
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < U; ++g) {
+        const int kn = k + (U + g) * kstep;
+        j[g] = kn < nk ? col[kn * kSliceRows] : 0;
+      }
+#pragma unroll
+      for (int g = 0; g < U; ++g)
+        if (k + g * kstep < nk) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) acc = fma(w[g][d], x[g][d], acc);
+        }
+    }
+    return join(acc, 0);
+  };
+  // the first slice's rows, and this lane's vector entries of it
+  const int fq0 = first < last ? a.m.slice_off[first] : 0;
+  const int fnk = first < last ? a.m.slice_off[first + 1] - fq0 : 0;
+  const int fv = vec && fnk > 0 ? row(first) : -1;
+  const size_t fo = fv >= 0 ? 3 * (size_t)fv + c : 0;
+  double fr = 0.0, fz = 0.0, fp = 0.0, fs = 0.0, fy = 0.0, fd = 0.0, fw = 0.0;
 
   // Diagonal blocks (minus the sum of the row's others, plus the mass), the
   // right-hand side, and z = r / diag(A).
   const bool rhs = a.finish != FIN_ADJOINT;
-  for (int s = s0; s < a.m.nslice; s += sstep) {
+  for (int s = first; s < last; s += sstep) {
     const int q0 = a.m.slice_off[s], nk = a.m.slice_off[s + 1] - q0;
     if (nk == 0) continue;
     const int v = row(s);
@@ -355,33 +403,38 @@ __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __
         b = a.gv[pl] + a.dt * a.gu[pl];
       }
       if (a.fresh) a.dinv[o] = di;
-      a.r[o] = b;
-      a.z[o] = b * di;
-      a.p[o] = 0.0;
-      a.s[o] = 0.0;
-      a.y[o] = 0.0;
+      const double z = b * di;
+      a.z[o] = z;
+      if (s == first) {
+        fr = b;
+        fz = z;
+        fd = di;
+      } else {
+        a.r[o] = b;
+        a.p[o] = 0.0;
+        a.s[o] = 0.0;
+        a.y[o] = 0.0;
+      }
     }
   }
   int status = EBB_OK, it = 0;
   double bb = 0.0, rr = 0.0, tol = 0.0;
-  bool ok = grid_wait(sh, a.bar, round);
+  grid_arrive(a.bar, round);
+  bool ok = grid_join(sh, a.bar, round);
   while (ok) {
     double sums[kSums] = {0.0, 0.0, 0.0};
-    for (int s = s0; s < a.m.nslice; s += sstep) {
+    if (SPLIT ? first < last : fnk > 0) {
+      fw = product(fq0, fnk);
+      if (fv >= 0) {
+        sums[0] = fr * fz;
+        sums[1] = fw * fz;
+        sums[2] = fr * fr;
+      }
+    }
+    for (int s = first + sstep; s < last; s += sstep) {
       const int q0 = a.m.slice_off[s], nk = a.m.slice_off[s + 1] - q0;
       if (nk == 0) continue;
-      double acc = 0.0;
-      const int* col = a.m.col + (size_t)q0 * kSliceRows + i;
-      const double* val = a.val + (size_t)q0 * 96 + lane;
-#pragma unroll 4
-      for (int k = k0; k < nk; k += kstep) {
-        const double* x = a.z + 3 * (size_t)col[k * kSliceRows];
-        const double x0 = x[0], x1 = x[1], x2 = x[2];
-        acc = fma(ld_stream(val + k * 96), x0, acc);
-        acc = fma(ld_stream(val + k * 96 + 32), x1, acc);
-        acc = fma(ld_stream(val + k * 96 + 64), x2, acc);
-      }
-      acc = join(acc, 0);
+      const double acc = product(q0, nk);
       const int v = vec ? row(s) : -1;
       if (v >= 0) {
         const size_t o = 3 * (size_t)v + c;
@@ -395,30 +448,41 @@ __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __
     ok = grid_sum(sh, sums, a.part, a.bar, round);
     if (!ok) break;
     rr = sh.tot[2];
-    if (it == 0) {
-      bb = rr;
-      if (threadIdx.x == 32) tol = a.rtol * sqrt(bb);
-    }
+    if (it == 0) bb = rr;
+    // The scalars, by one thread each: alpha and beta, the convergence test,
+    // and 1 / r.z for the next iteration (the divisions are FP64 chains).
+    const double rz = sh.tot[0];
     if (threadIdx.x == 0) {
-      const double rz = sh.tot[0];
-      const double beta = it > 0 ? rz * sh.scal[2] : 0.0;
-      const double pq = it > 0 ? sh.tot[1] - beta * (rz / sh.scal[0]) : sh.tot[1];
-      sh.scal[0] = rz / pq;
-      sh.scal[1] = beta;
-      sh.scal[2] = 1.0 / rz;
-      sh.scal[3] = pq;
+      double beta = 0.0, pq = sh.tot[1];
+      if (it > 0) {
+        beta = rz * sh.inv[~it & 1];
+        pq -= beta * (rz * (sh.pq * sh.inv[~it & 1]));   // 1 / alpha' = (p.Ap)' / (r.z)'
+      }
+      sh.pq = pq;
+      sh.alpha = rz / pq;
+      sh.beta = beta;
     } else if (threadIdx.x == 32) {
+      if (it == 0) tol = a.rtol * sqrt(bb);
       sh.active = it < a.max_iters && sqrt(rr) > tol;
+    } else if (threadIdx.x == 64) {
+      sh.inv[it & 1] = 1.0 / rz;
     }
     __syncthreads();
     if (!sh.active) break;
-    if (!(sh.scal[3] > 0.0)) {
+    if (!(sh.pq > 0.0)) {
       status = EBB_ERR_CG_BREAKDOWN;
       break;
     }
-    const double alpha = sh.scal[0], beta = sh.scal[1];
+    const double alpha = sh.alpha, beta = sh.beta;
+    const double zold = fz;
+    if (fv >= 0) {
+      fs = fma(beta, fs, fw);
+      fr = fma(-alpha, fs, fr);
+      fz = fr * fd;
+      a.z[fo] = fz;
+    }
     if (vec)
-      for (int s = s0; s < a.m.nslice; s += sstep) {
+      for (int s = first + sstep; s < last; s += sstep) {
         const int v = row(s);
         if (v < 0) continue;
         const size_t o = 3 * (size_t)v + c;
@@ -431,14 +495,17 @@ __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __
         a.z[o] = ri * a.dinv[o];
       }
     ++it;
-    ok = grid_wait(sh, a.bar, round);
+    grid_arrive(a.bar, round);
+    fp = fma(beta, fp, zold);
+    fy = fma(alpha, fp, fy);
+    ok = grid_join(sh, a.bar, round);
   }
   if (!ok) status = EBB_ERR_TIMEOUT;
   if (vec && ok)
-    for (int s = s0; s < a.m.nslice; s += sstep) {
+    for (int s = first; s < last; s += sstep) {
       const int v = row(s);
       if (v < 0) continue;
-      const double dv = a.y[3 * (size_t)v + c];
+      const double dv = s == first ? fy : a.y[3 * (size_t)v + c];
       const size_t pl = (size_t)c * a.nv + v;
       if (a.finish == FIN_STEP) {
         const double vi = a.v[pl] + dv;
@@ -496,15 +563,10 @@ cudaError_t launch_cg(const RowCgArgs& a, const PT* pin, int grid, cudaStream_t 
 }
 
 template <typename PT>
-cudaError_t solve(const RowCgArgs& a, const PT* pin, int nv, cudaStream_t st) {
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  nsm = std::min(std::max(nsm, 1), kMaxGrid);
-  const int slices = (nv + kSliceRows - 1) / kSliceRows;   // that hold rows
-  if (slices <= 3 * nsm) return launch_cg<kSplitThreads, true, PT>(a, pin, std::min(nsm, a.m.nslice), st);
-  return launch_cg<kPlainThreads, false, PT>(a, pin, nsm, st);
+cudaError_t solve(const RowCgArgs& a, const PT* pin, int grid, cudaStream_t st) {
+  const int slices = (a.nv + kSliceRows - 1) / kSliceRows;   // that hold rows
+  if (slices <= 3 * grid) return launch_cg<kSplitThreads, true, PT>(a, pin, grid, st);
+  return launch_cg<kPlainThreads, false, PT>(a, pin, grid, st);
 }
 
 // The step's buffers, in one allocation.  *fits is false when the device has
@@ -618,7 +680,7 @@ ebb_status_t row_step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v
   }
   ebb_status_t status = EBB_OK;
   if (forward) {
-    e = solve<PT>(ca, pin, nv, st);
+    e = solve<PT>(ca, pin, m.grid, st);
     if (e == cudaSuccess && vjp) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_check(ctx, e, "CG solve");
     if (vjp && s->host->status != EBB_OK)
@@ -633,7 +695,7 @@ ebb_status_t row_step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v
     ca.out = lam;
     ca.gu = vjp->gu;
     ca.gv = vjp->gv;
-    if (e == cudaSuccess) e = solve<PT>(ca, pin, nv, st);
+    if (e == cudaSuccess) e = solve<PT>(ca, pin, m.grid, st);
     if (e == cudaSuccess)
       e = launch_adjoint_map(tets, prm->mu, prm->lambda, u, lam, w, kl, xq, vjp->gmu, vjp->glam, prm->dt, st);
     if (e == cudaSuccess) {
