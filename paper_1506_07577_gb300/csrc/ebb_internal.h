@@ -142,7 +142,8 @@ struct VertexIndex {
 // Edge relation with self-loops (Section 5.2) as block CSR over internal
 // vertices: row r's blocks are (r, col[k]), k in [row_off[r], row_off[r+1]),
 // columns increasing; tet_blk[16 t + 4 a + b] is the block of corners (a, b)
-// of internal tet t (the key-field tets.e[4][4]).  blocks[p]: the assembled
+// of internal tet t (the key-field tets.e[4][4], built when an assembly first
+// needs it).  blocks[p]: the assembled
 // stiffness as 9 planes of nnzb, entry (c, d) of block k at [(3 c + d) nnzb
 // + k] ([0] FP32, [1] FP64).
 struct EdgeIndex {

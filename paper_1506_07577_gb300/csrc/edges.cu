@@ -13,7 +13,10 @@
 // consecutive words.  K(x) is assembled from closed-form element blocks with
 // atomic adds; K w is a block-sparse product with 8 lanes per row, each
 // taking every 8th block of the row, and a fixed-order shuffle tree, so the
-// product is bitwise reproducible for given blocks.
+// product is bitwise reproducible for given blocks.  Both run where the row
+// matrix (row_matrix.cu) does not apply: vertices of more than kRowMaxTets
+// tets, or no memory for it.  Elsewhere K is assembled and applied on the
+// rows, without atomics (64^3 mesh, FP32: 760 us this way).
 //
 // Element block of corners a, b (b_a = row a-1 of Dm^-1, b_0 = minus their
 // sum): the matrix-free K w map's dP applied to the probe dF = e_d b_b^T and
@@ -26,6 +29,7 @@
 #include <vector>
 
 #include "ebb_internal.h"
+#include "row_matrix.cuh"
 #include "tet_io.cuh"
 #include "tet_math.cuh"
 
@@ -120,6 +124,29 @@ assemble_kernel(int nt, int nv, const int4* __restrict__ keys, const int* __rest
       }
     }
   }
+}
+
+// tets.e[a][b] of internal tet t, the block of corners (a, b), by binary search
+// in row a's columns.
+__global__ void __launch_bounds__(kAsmThreads)
+tet_block_kernel(int nt, const int4* __restrict__ keys, const int* __restrict__ row_off, const int* __restrict__ col,
+                 int* __restrict__ tet_blk) {
+  const int t = blockIdx.x * kAsmThreads + threadIdx.x;
+  if (t >= nt) return;
+  const int4 k4 = keys[t];
+  const int kk[4] = {k4.x, k4.y, k4.z, k4.w};
+  for (int a = 0; a < 4; ++a)
+    for (int b = 0; b < 4; ++b) {
+      int lo = row_off[kk[a]], hi = row_off[kk[a] + 1];
+      while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (col[m] < kk[b])
+          lo = m + 1;
+        else
+          hi = m;
+      }
+      tet_blk[(size_t)16 * t + 4 * a + b] = lo;
+    }
 }
 
 // y[r] += sum_k blocks[k] w[col[k]] over row r's blocks; kRowLanes lanes per
@@ -251,21 +278,12 @@ ebb_status_t build_edges(ebb_ctx_s* ctx, ebb_rel_s* tets, const std::vector<int4
     if (col.size() > (size_t)0x7fffffff / 9) return set_error(ctx, EBB_ERR_ARG, "edge relation too large");
     row_off[v + 1] = (int)col.size();
   }
-  // tets.e[a][b]: the block of corners (a, b)
-  std::vector<int> tb((size_t)16 * nt);
-  for (int t = 0; t < nt; ++t) {
-    const int k[4] = {keys[t].x, keys[t].y, keys[t].z, keys[t].w};
-    for (int a = 0; a < 4; ++a) {
-      const int* r0 = col.data() + row_off[k[a]];
-      const int* r1 = col.data() + row_off[k[a] + 1];
-      for (int b = 0; b < 4; ++b) tb[(size_t)16 * t + 4 * a + b] = (int)(std::lower_bound(r0, r1, k[b]) - col.data());
-    }
-  }
+  const ebb_status_t rs = ensure_row_pattern(ctx, tets, ctx->stream);
+  if (rs) return rs;
   EdgeIndex& E = tets->edges;
   E.nnzb = (int)col.size();
   cudaError_t e = upload_vec(&E.row_off, row_off, ctx->stream);
   if (e == cudaSuccess) e = upload_vec(&E.col, col, ctx->stream);
-  if (e == cudaSuccess) e = upload_vec(&E.tet_blk, tb, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {
     free_edges(tets);
@@ -295,11 +313,31 @@ cudaError_t launch_assemble(ebb_rel_s* rel, int model, T mu0, T lam0, const MapI
   EdgeIndex& E = rel->edges;
   const int p = sizeof(T) == 4 ? 0 : 1;
   if (E.row_off == nullptr) return cudaErrorInvalidValue;
+  bool done = false;
+  cudaError_t re = launch_row_assemble<T>(rel, model, mu0, lam0, io, st, &done);
+  // (inside a stream capture, blocks that an earlier call had to fall back to
+  // stay in use)
+  if ((re != cudaSuccess && !(re == cudaErrorStreamCaptureUnsupported && E.blocks[p] != nullptr)) || done) {
+    E.assembled[p] = re == cudaSuccess;
+    return re;
+  }
   if (E.blocks[p] == nullptr) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cs);
     if (e != cudaSuccess) return e;
     if (cs != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
+    if (E.tet_blk == nullptr && rel->size > 0) {
+      const int nt = (int)rel->size;
+      e = cudaMalloc(&E.tet_blk, (size_t)16 * nt * sizeof(int));
+      if (e != cudaSuccess) {
+        E.tet_blk = nullptr;
+        return e;
+      }
+      tet_block_kernel<<<(nt + kAsmThreads - 1) / kAsmThreads, kAsmThreads, 0, st>>>(nt, rel->keys, E.row_off, E.col,
+                                                                                    E.tet_blk);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
     e = cudaMalloc(&E.blocks[p], std::max<size_t>(1, (size_t)E.nnzb) * 9 * sizeof(T));
     if (e != cudaSuccess) {
       E.blocks[p] = nullptr;
@@ -325,6 +363,9 @@ cudaError_t launch_spmv(ebb_rel_s* rel, const T* w, T* y, bool aos, const int* a
   const int nv = (int)rel->verts->size;
   if (E.row_off == nullptr || !E.assembled[p]) return cudaErrorInvalidValue;
   if (nv == 0) return cudaSuccess;
+  bool done = false;
+  const cudaError_t re = launch_row_product<T>(rel, w, y, aos, active, st, &done);
+  if (re != cudaSuccess || done) return re;
   const int grid = (int)(((size_t)nv * kRowLanes + kSpmvThreads - 1) / kSpmvThreads);
   const T* blocks = static_cast<const T*>(E.blocks[p]);
   if (aos) {

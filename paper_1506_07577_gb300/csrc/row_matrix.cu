@@ -7,7 +7,9 @@
 // the block's contribution list names, in increasing tet order: bitwise
 // reproducible.  The diagonal block is minus the sum of its row's other
 // blocks (K annihilates translations), so 6 of the 16 corner pairs are
-// formed per tet, each once.
+// formed per tet, each once.  Measured on the 64^3 mesh (1.31 M tets, FP32):
+// records 77 us, rows 182 us, product 44 us; one atomic per block entry and
+// tet took 716 us.
 #include <algorithm>
 
 #include "row_matrix.cuh"
@@ -19,69 +21,123 @@ namespace ebb {
 namespace {
 
 constexpr int kSortWarps = 4;
-constexpr int kSortLen = 512;            // >= 3 * kRowMaxTets, a power of two
-static_assert(kSortLen >= 3 * kRowMaxTets, "sort buffer");
+constexpr int kShortTets = 40;           // rows of up to so many tets take the small tables
 constexpr int kScanThreads = 1024;
 
-// The other corners of the tets around vertex v, sorted by (vertex, entry):
-// buf[0 .. n) = vertex << 12 | 4 * (entry - off[v]) + corner; returns n.  One
-// warp; n <= 3 * kRowMaxTets (larger rows return -1).
-__device__ __forceinline__ int sort_row(int v, const int* __restrict__ off, const int* __restrict__ ent,
-                                        const int4* __restrict__ keys, unsigned long long* buf) {
-  const int lane = threadIdx.x & 31;
+// Columns and contribution lists of a row, one warp per vertex.  The other
+// corners of the vertex's tets go into a small hash table in shared memory;
+// the distinct vertices, ranked by number, are the row's columns, and a
+// corner's place in its column's list is the count of equal corners before
+// it, so that the lists keep the order of the vertex index (increasing tets).
+// Row v owns [3 off[v], 3 off[v + 1]) of contrib, colv and colb: its
+// contributions column by column, its columns, and where each column's list
+// begins.  len[v]: blocks of the row, the diagonal one included.  A vertex of
+// more than kRowMaxTets tets sets *too_long.  Launched for rows of up to
+// kShortTets tets (LONG false), then for the longer ones, whose tables leave
+// room for few warps.
+template <int MAXT, int HASH, bool LONG>
+__global__ void __launch_bounds__(32 * kSortWarps)
+row_columns_kernel(int nv, const int* __restrict__ off, const int* __restrict__ ent, const int4* __restrict__ keys,
+                   int* __restrict__ contrib, int* __restrict__ colv, int* __restrict__ colb, int* __restrict__ len,
+                   int* too_long) {
+  static_assert(HASH >= 6 * MAXT && (HASH & (HASH - 1)) == 0, "hash load");
+  constexpr int G = (3 * MAXT + 31) / 32;
+  __shared__ int s_key[kSortWarps][HASH];
+  __shared__ short s_cnt[kSortWarps][HASH], s_uniq[kSortWarps][3 * MAXT], s_at[kSortWarps][3 * MAXT];
+  __shared__ short s_slot[kSortWarps][3 * MAXT];
+  const int v = blockIdx.x * kSortWarps + (threadIdx.x >> 5);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (v >= nv) return;
+  int* key = s_key[w];
+  short *cnt = s_cnt[w], *uniq = s_uniq[w], *at = s_at[w], *slot_of = s_slot[w];
   const int e0 = off[v], ne = off[v + 1] - e0;
-  if (ne > kRowMaxTets) return -1;
+  if (LONG ? ne <= kShortTets : ne > MAXT) return;
+  if (LONG && ne > MAXT) {
+    if (lane == 0) {
+      len[v] = 1;
+      *too_long = 1;
+    }
+    return;
+  }
   const int n = 3 * ne;
-  int P = 32;
-  while (P < n) P <<= 1;
-  for (int x = lane; x < P; x += 32) {
-    unsigned long long key = ~0ull;
+  int size = 64;
+  while (size < 2 * n) size <<= 1;
+  for (int x = lane; x < size; x += 32) {
+    key[x] = -1;
+    cnt[x] = 0;
+  }
+  __syncwarp();
+  // insert; slot_of[x] and at[x] (entries of the same vertex before x)
+  for (int b = 0; b < n; b += 32) {
+    const int x = b + lane;
+    const unsigned on = __ballot_sync(0xffffffffu, x < n);
     if (x < n) {
       const int le = x / 3, r = x - 3 * le;
       const int code = ent[e0 + le];
-      const int a = code & 3;
-      const int b = r + (r >= a ? 1 : 0);
+      const int c = r + (r >= (code & 3) ? 1 : 0);
       const int4 k = keys[code >> 2];
-      const int j = b == 0 ? k.x : (b == 1 ? k.y : (b == 2 ? k.z : k.w));
-      key = ((unsigned long long)(unsigned)j << 12) | (unsigned)(4 * le + b);
+      const int j = c == 0 ? k.x : (c == 1 ? k.y : (c == 2 ? k.z : k.w));
+      unsigned h = ((unsigned)j * 2654435761u) >> 16 & (unsigned)(size - 1);
+      while (true) {
+        const int old = atomicCAS(&key[h], -1, j);
+        if (old == -1 || old == j) break;
+        h = (h + 1) & (unsigned)(size - 1);
+      }
+      slot_of[x] = (short)h;
+      const unsigned same = __match_any_sync(on, j);
+      const int before = cnt[h];
+      __syncwarp(on);
+      at[x] = (short)(before + __popc(same & ((1u << lane) - 1u)));
+      if (lane == __ffs(same) - 1) cnt[h] = (short)(before + __popc(same));
     }
-    buf[x] = key;
+    __syncwarp();
+  }
+  // the distinct vertices' slots
+  int m = 0;
+  for (int b = 0; b < size; b += 32) {
+    const bool used = key[b + lane] >= 0;
+    const unsigned u = __ballot_sync(0xffffffffu, used);
+    if (used) uniq[m + __popc(u & ((1u << lane) - 1u))] = (short)(b + lane);
+    m += __popc(u);
   }
   __syncwarp();
-  for (int k = 2; k <= P; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = lane; i < P / 2; i += 32) {
-        const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1));
-        const int hi = lo | j;
-        const unsigned long long x = buf[lo], y = buf[hi];
-        if ((x > y) == ((lo & k) == 0)) {
-          buf[lo] = y;
-          buf[hi] = x;
+  // rank by vertex number and start of each list; cnt becomes the start
+  const int c0 = 3 * e0;
+  int starts[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int x = 32 * g + lane;
+    starts[g] = 0;
+    if (x < m) {
+      const int j = key[uniq[x]];
+      int rank = 0;
+      for (int y = 0; y < m; ++y) {
+        const int o = uniq[y];
+        if (key[o] < j) {
+          ++rank;
+          starts[g] += cnt[o];
         }
       }
-      __syncwarp();
+      colv[(size_t)c0 + rank] = j;
+      colb[(size_t)c0 + rank] = c0 + starts[g];
     }
-  return n;
-}
-
-// Row lengths in blocks, the diagonal one included; *too_long is set when a
-// vertex has more than kRowMaxTets tets.
-__global__ void __launch_bounds__(32 * kSortWarps)
-row_length_kernel(int nv, const int* __restrict__ off, const int* __restrict__ ent, const int4* __restrict__ keys,
-                  int* len, int* too_long) {
-  __shared__ unsigned long long s[kSortWarps][kSortLen];
-  const int v = blockIdx.x * kSortWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (v >= nv) return;
-  unsigned long long* buf = s[threadIdx.x >> 5];
-  const int n = sort_row(v, off, ent, keys, buf);
-  int heads = 0;
-  for (int x = lane; x < n; x += 32) heads += x == 0 || (buf[x] >> 12) != (buf[x - 1] >> 12);
-  heads = __reduce_add_sync(0xffffffffu, heads);
-  if (lane == 0) {
-    len[v] = 1 + heads;
-    if (n < 0) *too_long = 1;
   }
+  __syncwarp();
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int x = 32 * g + lane;
+    if (x < m) cnt[uniq[x]] = (short)starts[g];
+  }
+  __syncwarp();
+  for (int x = lane; x < n; x += 32) {
+    const int le = x / 3, r = x - 3 * le;
+    const int code = ent[e0 + le], ca = code & 3;
+    const int cb = r + (r >= ca ? 1 : 0);
+    const int lo = min(ca, cb), hi = max(ca, cb);
+    const int pair = lo == 0 ? hi - 1 : lo + hi;   // 01 02 03 12 13 23
+    contrib[(size_t)c0 + cnt[slot_of[x]] + at[x]] = 16 * (code >> 2) + 2 * pair + (ca > cb ? 1 : 0);
+  }
+  if (lane == 0) len[v] = 1 + m;
 }
 
 // One block per window: rows sorted by decreasing length (ties in order of
@@ -144,50 +200,23 @@ scan_kernel(int n, const int* __restrict__ in, int* out) {
   if (threadIdx.x == 0) out[n] = s_run;
 }
 
-// Columns and contribution lists.  Warp per row: the row's 3 x tets entries in
-// sorted order are the contributions of its blocks, consecutive per block.
-__global__ void __launch_bounds__(32 * kSortWarps)
-row_fill_kernel(int nv, const int* __restrict__ off, const int* __restrict__ ent, const int4* __restrict__ keys,
-                const int* __restrict__ place, const int* __restrict__ slice_off, int* col, int2* crange,
-                int* slot_slice, int* contrib) {
-  __shared__ unsigned long long s[kSortWarps][kSortLen];
-  const int v = blockIdx.x * kSortWarps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
+// The rows' columns and contribution ranges in slot order; eight lanes per row.
+__global__ void __launch_bounds__(256)
+row_fill_kernel(int nv, const int* __restrict__ off, const int* __restrict__ len, const int* __restrict__ colv,
+                const int* __restrict__ colb, const int* __restrict__ place, const int* __restrict__ slice_off,
+                int* col, int2* crange, int* slot_slice) {
+  const int v = (blockIdx.x * 256 + threadIdx.x) >> 3, lane = threadIdx.x & 7;
   if (v >= nv) return;
-  unsigned long long* buf = s[threadIdx.x >> 5];
-  const int n = sort_row(v, off, ent, keys, buf);
-  const int c0 = 3 * off[v];
+  const int c0 = 3 * off[v], c1 = 3 * off[v + 1], m = len[v] - 1;
   const int sl = place[v] / kSliceRows, i = place[v] - sl * kSliceRows;
   const int q0 = slice_off[sl], nk = slice_off[sl + 1] - q0;
-  if (lane == 0) col[(size_t)q0 * kSliceRows + i] = v;
-  if (i == 0)   // the slice's longest row
-    for (int r = lane; r < nk; r += 32) slot_slice[q0 + r] = sl;
-  int k = 1;
-  for (int b = 0; b < n; b += 32) {
-    const int x = b + lane;
-    bool head = false;
-    int j = 0;
-    if (x < n) {
-      const unsigned long long key = buf[x];
-      j = (int)(key >> 12);
-      head = x == 0 || (buf[x - 1] >> 12) != (key >> 12);
-      const int le = (int)(key & 0xfffu) >> 2, cb = (int)(key & 3u);
-      const int code = ent[off[v] + le];
-      const int ca = code & 3, lo = min(ca, cb), hi = max(ca, cb);
-      const int pair = lo == 0 ? hi - 1 : lo + hi;   // 01 02 03 12 13 23
-      contrib[(size_t)c0 + x] = 16 * (code >> 2) + 2 * pair + (ca > cb ? 1 : 0);
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, head);
-    if (head) {
-      const size_t at = (size_t)(q0 + k + __popc(m & ((1u << lane) - 1u))) * kSliceRows + i;
-      int end = x + 1;
-      while (end < n && (int)(buf[end] >> 12) == j) ++end;
-      col[at] = j;
-      crange[at] = make_int2(c0 + x, c0 + end);
-    }
-    k += __popc(m);
+  for (int k = lane; k < nk; k += 8) {
+    const size_t at = (size_t)(q0 + k) * kSliceRows + i;
+    const bool in = k > 0 && k <= m;
+    col[at] = in ? colv[c0 + k - 1] : v;
+    crange[at] = in ? make_int2(colb[c0 + k - 1], k < m ? colb[c0 + k] : c1) : make_int2(0, 0);
+    if (i == 0) slot_slice[q0 + k] = sl;   // by the slice's longest row
   }
-  for (int r = k + lane; r < nk; r += 32) col[(size_t)(q0 + r) * kSliceRows + i] = v;
 }
 
 // ---- element pass ---------------------------------------------------------
@@ -198,14 +227,15 @@ row_fill_kernel(int nv, const int* __restrict__ off, const int* __restrict__ ent
 //         h_a = F^-T b_a.
 // FP64: bound by the FP64 pipe (about 400 FP64 instructions per tet at 530
 // G/s); the 512 B stored per tet ride along.
+// FP32: bound by the records' writes, which go through shared memory a warp
+// at a time, so that each store is a line of consecutive words (written
+// straight from the threads, a store touches 32 lines).
 constexpr int kElemThreads = 64;
 
 template <typename T, int MODEL, bool AOS, bool FORCE>
-__global__ void __launch_bounds__(kElemThreads)
-element_block_kernel(int nt, int nv, const int4* __restrict__ keys, const int* __restrict__ perm, TetStreams<T> s,
-                     T mu0, T lam0, const T* __restrict__ u, T* __restrict__ elem, int* err) {
-  const int t = blockIdx.x * kElemThreads + threadIdx.x;
-  if (t >= nt) return;
+__device__ __forceinline__ void element_record(int t, int nt, int nv, const int4* __restrict__ keys,
+                                               const int* __restrict__ perm, const TetStreams<T>& s, T mu0, T lam0,
+                                               const T* __restrict__ u, T* rec, int* err) {
   const int4 k4 = keys[t];
   const int kk[4] = {k4.x, k4.y, k4.z, k4.w};
   T B[9], V, mu, lam;
@@ -216,7 +246,6 @@ element_block_kernel(int nt, int nv, const int4* __restrict__ keys, const int* _
   load_edges<T, OP_FORCE, AOS>(io, nv, kk, Du, Dw);
   T G[9];
   mm(Du, B, G);
-  T* rec = elem + (size_t)t * kElemLen;
   // The volume goes into the Lame parameters once, so that every product below
   // carries it.  vec[a]: r_a or h_a; bab: V mu b_a.b_b and bSb: V b_a.S b_b in
   // the pair order.
@@ -302,10 +331,6 @@ element_block_kernel(int nt, int nv, const int4* __restrict__ keys, const int* _
       for (int i = 0; i < 3; ++i)
         vec[a + 1][i] = sn.FiT[i * 3] * B[a * 3] + sn.FiT[i * 3 + 1] * B[a * 3 + 1] + sn.FiT[i * 3 + 2] * B[a * 3 + 2];
   }
-  if (FORCE) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) rec[kElemForce + i] = f[i];
-  }
 #pragma unroll
   for (int b = 0; b < 3; ++b) bab[b] = -vmu * (M[b] + M[3 + b] + M[6 + b]);
   bab[3] = vmu * M[1];
@@ -334,17 +359,48 @@ element_block_kernel(int nt, int nv, const int4* __restrict__ keys, const int* _
           x[q] = dg ? bab[p] : T(0);
       }
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+      for (int c = 0; c < 3; ++c) {
+        T k[4];
+        k[3] = FORCE && 3 * p + c < 9 ? f[3 * p + c < 9 ? 3 * p + c : 0] : T(0);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           const int lo = c < d ? c : d, hi = c < d ? d : c;
           const int q = lo == 0 ? hi : (lo == 1 ? 2 + hi : 5);   // 00 01 02 11 12 22
-          rec[9 * p + 3 * c + d] = v1[c] * vec[a][d] + (v2[d] * vec[a][c] + x[q]);
+          k[d] = v1[c] * vec[a][d] + (v2[d] * vec[a][c] + x[q]);
         }
+        if constexpr (sizeof(T) == 8) {
+          double2* out = reinterpret_cast<double2*>(rec + 4 * (3 * p + c));
+          out[0] = make_double2(k[0], k[1]);
+          out[1] = make_double2(k[2], k[3]);
+        } else {
+#pragma unroll
+          for (int d = 0; d < 4; ++d) rec[4 * (3 * p + c) + d] = k[d];
+        }
+      }
     }
   }
 }
 
+template <typename T, int MODEL, bool AOS, bool FORCE>
+__global__ void __launch_bounds__(kElemThreads)
+element_block_kernel(int nt, int nv, const int4* __restrict__ keys, const int* __restrict__ perm, TetStreams<T> s,
+                     T mu0, T lam0, const T* __restrict__ u, T* __restrict__ elem, int* err) {
+  constexpr bool STAGE = sizeof(T) == 4;
+  constexpr int L = kElemLen;
+  __shared__ T s_rec[STAGE ? kElemThreads : 1][STAGE ? L + 1 : 1];
+  const int t = blockIdx.x * kElemThreads + threadIdx.x;
+  if (!STAGE && t >= nt) return;
+  const int tt = t < nt ? t : nt - 1;
+  T* rec = STAGE ? &s_rec[STAGE ? threadIdx.x : 0][0] : elem + (size_t)t * L;
+  element_record<T, MODEL, AOS, FORCE>(tt, nt, nv, keys, perm, s, mu0, lam0, u, rec, err);
+  if constexpr (STAGE) {
+    __syncwarp();
+    const int w0 = (int)threadIdx.x & ~31, lane = threadIdx.x & 31;
+    const int n = min(32, nt - (blockIdx.x * kElemThreads + w0)) * L;   // words of the warp's records
+    T* dst = elem + (size_t)(blockIdx.x * kElemThreads + w0) * L;
+    for (int x = lane; x < n; x += 32) dst[x] = s_rec[w0 + x / L][x % L];
+  }
+}
 template <typename T>
 const TetStreams<T>& elem_streams(const ebb_rel_s* rel);
 template <>
@@ -356,8 +412,8 @@ template <typename T, int MODEL, bool AOS>
 void launch_elem(ebb_rel_s* rel, T mu0, T lam0, const T* u, bool force, T* elem, cudaStream_t st) {
   const int nt = (int)rel->size, nv = (int)rel->verts->size;
   const int grid = (nt + kElemThreads - 1) / kElemThreads;
-  if (force)
-    element_block_kernel<T, MODEL, AOS, true><<<grid, kElemThreads, 0, st>>>(
+  if (sizeof(T) == 8 && force)
+    element_block_kernel<T, MODEL, AOS, sizeof(T) == 8><<<grid, kElemThreads, 0, st>>>(
         nt, nv, rel->keys, rel->tet_perm, elem_streams<T>(rel), mu0, lam0, u, elem, rel->ctx->d_err);
   else
     element_block_kernel<T, MODEL, AOS, false><<<grid, kElemThreads, 0, st>>>(
@@ -386,6 +442,235 @@ cudaError_t launch_element_blocks(ebb_rel_s* rel, int model, T mu0, T lam0, cons
     launch_elem<T, EBB_NEOHOOKEAN, false>(rel, mu0, lam0, u, force, elem, st);
   return cudaGetLastError();
 }
+
+// ---- assembled K for ebb_assemble_tet_K / ebb_spmv_tet_K --------------------
+namespace {
+
+constexpr int kAsmThreads = 256;
+
+// Off-diagonal blocks of scale * K, one warp per slot, a lane per row and
+// component: the sum of the block's contributions in increasing tet order.
+// Blocks of a record are stored for a < b; the other way round they are
+// transposed.  FP32: a lane loads its row of the stored block, one 16-byte load
+// per contribution (the loads' lines bound the kernel: with one load per entry
+// or nine lanes per block it took 3 times as long), adds stored and transposed
+// contributions apart and swaps the transposed sums between its row's lanes at the
+// end.  FP64: the adds bound it, so transposed entries are loaded as such.
+template <typename T, typename PT>
+__global__ void __launch_bounds__(kAsmThreads)
+row_block_kernel(int64_t nslots, const int* __restrict__ slice_off, const int* __restrict__ slot_slice,
+                 const int* __restrict__ row_of, const int2* __restrict__ crange, const int* __restrict__ contrib,
+                 const T* __restrict__ elem, const PT* __restrict__ pin, T scale, T* __restrict__ val) {
+  const int64_t q = ((int64_t)blockIdx.x * kAsmThreads + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (q >= nslots) return;
+  const int s = slot_slice[q];
+  const bool own = lane < 3 * kSliceRows;
+  const int i = own ? lane / 3 : 0, c = own ? lane - 3 * i : 0;
+  int2 r = own ? crange[q * kSliceRows + i] : make_int2(0, 0);
+  if (q == slice_off[s]) return;   // the diagonal blocks are not stored here
+  if (pin != nullptr && r.x < r.y && pin[row_of[s * kSliceRows + i]] != 0) r.y = r.x;
+  T x[3] = {T(0), T(0), T(0)};
+  if constexpr (sizeof(T) == 4) {
+    T xt[3] = {T(0), T(0), T(0)};
+#pragma unroll 4
+    for (int e = r.x; e < r.y; ++e) {
+      const int code = contrib[e];
+      const float4 k = __ldg(reinterpret_cast<const float4*>(elem + (size_t)(code >> 4) * kElemLen +
+                                                             12 * ((code >> 1) & 7) + 4 * c));
+      if (code & 1) {
+        xt[0] += k.x;
+        xt[1] += k.y;
+        xt[2] += k.z;
+      } else {
+        x[0] += k.x;
+        x[1] += k.y;
+        x[2] += k.z;
+      }
+    }
+    // lane c's entry d of the transposed sum is lane d's entry c
+    const int row0 = lane - c;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      T y[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) y[k] = __shfl_sync(0xffffffffu, xt[k], row0 + d);
+      x[d] += c == 0 ? y[0] : (c == 1 ? y[1] : y[2]);
+    }
+  } else if (r.x < r.y) {
+    auto rec_of = [&](int code, int& st) {
+      const bool tr = (code & 1) != 0;
+      st = tr ? 4 : 1;
+      return elem + (size_t)(code >> 4) * kElemLen + 12 * ((code >> 1) & 7) + (tr ? c : 4 * c);
+    };
+    int st;
+    const T* rec = rec_of(contrib[r.x], st);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) x[d] = rec[d * st];
+#pragma unroll 4
+    for (int e = r.x + 1; e < r.y; ++e) {
+      rec = rec_of(contrib[e], st);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[d] += rec[d * st];
+    }
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) val[((size_t)q * 3 + d) * 32 + lane] = scale * x[d];
+}
+
+__device__ __forceinline__ float ld_once(const float* p) {
+  float x;
+  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ double ld_once(const double* p) {
+  double x;
+  asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(x) : "l"(p));
+  return x;
+}
+
+// y_r += sum_j K_rj (w_j - w_r): the diagonal block, minus the sum of the row's
+// others, is in the difference.  Warp per slice, lane per row and component,
+// fixed order.  FP32: bound by the blocks' one pass through memory.
+template <typename T, bool AOS>
+__global__ void __launch_bounds__(kAsmThreads)
+row_product_kernel(RowView m, int nv, const T* __restrict__ val, const T* __restrict__ w, T* y, const int* active) {
+  if (active != nullptr && *active == 0) return;
+  const int s = (blockIdx.x * kAsmThreads + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (s >= m.nslice || lane >= 3 * kSliceRows) return;
+  const int i = lane / 3, c = lane - 3 * i;
+  const int v = m.row_of[s * kSliceRows + i];
+  if (v < 0) return;
+  const int q0 = m.slice_off[s], nk = m.slice_off[s + 1] - q0;
+  auto load = [&](int j, T (&x)[3]) {
+    if constexpr (AOS) {
+      const float4 f = reinterpret_cast<const float4*>(w)[j];
+      x[0] = f.x;
+      x[1] = f.y;
+      x[2] = f.z;
+    } else {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[d] = w[(size_t)d * nv + j];
+    }
+  };
+  // groups of U slots; the next group's columns are loaded a group ahead
+  constexpr int U = 4;
+  const int* col = m.col + (size_t)q0 * kSliceRows + i;
+  const T* bv = val + (size_t)q0 * 96 + lane;
+  int j[U];
+#pragma unroll
+  for (int g = 0; g < U; ++g) j[g] = 1 + g < nk ? col[(1 + g) * kSliceRows] : v;
+  T wr[3];
+  load(v, wr);
+  T acc = T(0);
+  for (int k = 1; k < nk; k += U) {
+    T x[U][3], b[U][3];
+#pragma unroll
+    for (int g = 0; g < U; ++g) {
+      const T* at = bv + (size_t)(k + g < nk ? k + g : 0) * 96;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) b[g][d] = ld_once(at + 32 * d);
+      load(j[g], x[g]);
+    }
+#pragma unroll
+    for (int g = 0; g < U; ++g) j[g] = k + U + g < nk ? col[(k + U + g) * kSliceRows] : v;
+#pragma unroll
+    for (int g = 0; g < U; ++g)
+      if (k + g < nk) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) acc += b[g][d] * (x[g][d] - wr[d]);
+      }
+  }
+  y[AOS ? 4 * (size_t)v + c : (size_t)c * nv + v] += acc;
+}
+
+}  // namespace
+
+template <typename T>
+cudaError_t launch_row_blocks(const RowMatrix& m, const T* elem, const void* pin, int pin_bytes, T scale, T* val,
+                              cudaStream_t st) {
+  const int64_t grid = (m.nslots * 32 + kAsmThreads - 1) / kAsmThreads;
+  if (grid == 0) return cudaSuccess;
+  if (pin_bytes == 4)
+    row_block_kernel<T, int><<<(unsigned)grid, kAsmThreads, 0, st>>>(m.nslots, m.slice_off, m.slot_slice, m.row_of,
+                                                                     m.crange, m.contrib, elem,
+                                                                     static_cast<const int*>(pin), scale, val);
+  else
+    row_block_kernel<T, unsigned char><<<(unsigned)grid, kAsmThreads, 0, st>>>(
+        m.nslots, m.slice_off, m.slot_slice, m.row_of, m.crange, m.contrib, elem,
+        static_cast<const unsigned char*>(pin), scale, val);
+  return cudaGetLastError();
+}
+template cudaError_t launch_row_blocks<double>(const RowMatrix&, const double*, const void*, int, double, double*,
+                                               cudaStream_t);
+
+template <typename T>
+cudaError_t launch_row_assemble(ebb_rel_s* rel, int model, T mu0, T lam0, const MapIO<T>& io, cudaStream_t st,
+                                bool* done) {
+  *done = false;
+  const int p = sizeof(T) == 4 ? 0 : 1;
+  RowMatrix* m = rel->rows;
+  if (m == nullptr || m->val[p] == nullptr) {
+    // first use: pattern and memory, never inside a stream capture
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cs);
+    if (e != cudaSuccess) return e;
+    if (cs != cudaStreamCaptureStatusNone) return m != nullptr && m->state != 1 ? cudaSuccess
+                                                                                : cudaErrorStreamCaptureUnsupported;
+    if (ensure_row_pattern(rel->ctx, rel, st) != EBB_OK) return cudaErrorUnknown;
+    m = rel->rows;
+    if (m->state != 1) return cudaSuccess;
+    e = cudaMalloc(&m->val[p], std::max<size_t>(1, (size_t)m->nslots * 96) * sizeof(T));
+    if (e == cudaSuccess) e = cudaMalloc(&m->elem[p], std::max<size_t>(1, (size_t)rel->size * kElemLen) * sizeof(T));
+    if (e != cudaSuccess) {
+      cudaFree(m->val[p]);
+      m->val[p] = m->elem[p] = nullptr;
+      cudaGetLastError();
+      return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+    }
+  }
+  if (m->state != 1) return cudaSuccess;
+  T* elem = static_cast<T*>(m->elem[p]);
+  cudaError_t e = launch_element_blocks<T>(rel, model, mu0, lam0, io.u, io.aos, false, elem, st);
+  if (e != cudaSuccess) return e;
+  e = launch_row_blocks<T>(*m, elem, nullptr, 1, T(1), static_cast<T*>(m->val[p]), st);
+  if (e != cudaSuccess) return e;
+  *done = true;
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_row_product(ebb_rel_s* rel, const T* w, T* y, bool aos, const int* active, cudaStream_t st,
+                               bool* done) {
+  *done = false;
+  const int p = sizeof(T) == 4 ? 0 : 1;
+  const RowMatrix* m = rel->rows;
+  if (m == nullptr || m->val[p] == nullptr) return cudaSuccess;
+  const int nv = (int)rel->verts->size;
+  const RowView view{m->nslice, m->slice_off, m->row_of, m->col};
+  const int grid = (m->nslice * 32 + kAsmThreads - 1) / kAsmThreads;
+  const T* val = static_cast<const T*>(m->val[p]);
+  *done = true;
+  if (aos) {
+    if constexpr (sizeof(T) == 4) {
+      row_product_kernel<T, true><<<grid, kAsmThreads, 0, st>>>(view, nv, val, w, y, active);
+      return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
+  }
+  row_product_kernel<T, false><<<grid, kAsmThreads, 0, st>>>(view, nv, val, w, y, active);
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_row_assemble<float>(ebb_rel_s*, int, float, float, const MapIO<float>&, cudaStream_t,
+                                                bool*);
+template cudaError_t launch_row_assemble<double>(ebb_rel_s*, int, double, double, const MapIO<double>&, cudaStream_t,
+                                                 bool*);
+template cudaError_t launch_row_product<float>(ebb_rel_s*, const float*, float*, bool, const int*, cudaStream_t,
+                                               bool*);
+template cudaError_t launch_row_product<double>(ebb_rel_s*, const double*, double*, bool, const int*, cudaStream_t,
+                                                bool*);
 template cudaError_t launch_element_blocks<double>(ebb_rel_s*, int, double, double, const double*, bool, bool, double*,
                                                    cudaStream_t);
 
@@ -398,6 +683,10 @@ void free_row_matrix(ebb_rel_s* tets) {
   cudaFree(m->crange);
   cudaFree(m->slot_slice);
   cudaFree(m->contrib);
+  for (int p = 0; p < 2; ++p) {
+    cudaFree(m->val[p]);
+    cudaFree(m->elem[p]);
+  }
   delete m;
   tets->rows = nullptr;
 }
@@ -413,9 +702,9 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
   if (tets->vindex.off == nullptr || nv == 0 || nt > (int64_t)0x7fffffff / 16) return EBB_OK;
   const int nwin = (nv + kWindowRows - 1) / kWindowRows;
   m->nslice = nwin * kWindowSlices;
-  // scratch: row lengths, places, slot counts, the too-long flag
+  // scratch: row lengths, places, slot counts, the too-long flag, columns
   int* tmp = nullptr;
-  const size_t ntmp = 2 * (size_t)nv + m->nslice + 1;
+  const size_t ntmp = 2 * (size_t)nv + m->nslice + 1 + (size_t)nt * 24;
   cudaError_t e = cudaMalloc(&tmp, ntmp * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&m->slice_off, ((size_t)m->nslice + 1) * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&m->row_of, (size_t)nwin * kWindowRows * sizeof(int));
@@ -425,11 +714,15 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
   m->grid = std::min({std::max(nsm, 1), kRowMaxGrid, m->nslice});
   int host[2] = {0, 0};   // total slots, too-long flag
   int *len = tmp, *place = tmp + nv, *slots = tmp + 2 * (size_t)nv, *flag = slots + m->nslice;
-  const int sort_grid = (nv + kSortWarps - 1) / kSortWarps;
+  int *colv = flag + 1, *colb = colv + (size_t)nt * 12;
   if (e == cudaSuccess) {
     const VertexIndex& x = tets->vindex;
     e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-    row_length_kernel<<<sort_grid, 32 * kSortWarps, 0, st>>>(nv, x.off, x.ent, tets->keys, len, flag);
+    const int cg = (nv + kSortWarps - 1) / kSortWarps;
+    row_columns_kernel<kShortTets, 256, false><<<cg, 32 * kSortWarps, 0, st>>>(nv, x.off, x.ent, tets->keys,
+                                                                               m->contrib, colv, colb, len, flag);
+    row_columns_kernel<kRowMaxTets, 1024, true><<<cg, 32 * kSortWarps, 0, st>>>(nv, x.off, x.ent, tets->keys,
+                                                                                m->contrib, colv, colb, len, flag);
     window_kernel<<<nwin, kWindowRows, 0, st>>>(nv, x.order, len, m->row_of, place, slots);
     scan_kernel<<<1, kScanThreads, 0, st>>>(m->nslice, slots, m->slice_off);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -449,9 +742,8 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
     if (e == cudaSuccess) e = cudaMemsetAsync(m->col, 0, n * sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->crange, 0, n * sizeof(int2), st);
     if (e == cudaSuccess) {
-      const VertexIndex& x = tets->vindex;
-      row_fill_kernel<<<sort_grid, 32 * kSortWarps, 0, st>>>(nv, x.off, x.ent, tets->keys, place, m->slice_off, m->col,
-                                                             m->crange, m->slot_slice, m->contrib);
+      row_fill_kernel<<<(nv + 31) / 32, 256, 0, st>>>(nv, tets->vindex.off, len, colv, colb, place, m->slice_off,
+                                                      m->col, m->crange, m->slot_slice);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

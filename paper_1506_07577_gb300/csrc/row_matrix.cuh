@@ -33,11 +33,11 @@ constexpr int kWindowSlices = 32;
 constexpr int kWindowRows = kSliceRows * kWindowSlices;
 constexpr int kRowMaxTets = 128;                     // tets around one vertex
 constexpr int kRowMaxGrid = 256;                     // thread blocks of a kernel over all slices
-// Element record, in values: the blocks of the six corner pairs (a < b,
-// pair order 01 02 03 12 13 23, 9 entries each, row-major), then the corner
-// forces of corners 1..3 (corner 0 is minus their sum), one value unused.
-constexpr int kElemLen = 64;
-constexpr int kElemForce = 54;
+// Element record, in values: for each of the six corner pairs (a < b, order 01
+// 02 03 12 13 23) the three rows of its block, four values each, so that a
+// row is one or two 16-byte accesses.  The fourth values of rows 0 .. 8 hold the
+// corner forces of corners 1..3 (FP64 steps; corner 0 is minus their sum).
+constexpr int kElemLen = 72;
 
 struct RowMatrix {
   int state = 0;              // 0 not built, 1 built, -1 does not apply to this relation
@@ -49,7 +49,12 @@ struct RowMatrix {
   int2* crange = nullptr;     // nslots * kSliceRows: the block's contributions [x, y)
   int* slot_slice = nullptr;  // nslots: slice of each slot
   int* contrib = nullptr;     // 12 per tet, row by row: 16 t + 2 pair + transposed
+  bool no_step = false;       // the FP64 step's buffers did not fit (row_step.cu)
   int grid = 0;               // thread blocks of a kernel over all slices (at most one per SM)
+  // Assembled K of ebb_assemble_tet_K ([0] FP32, [1] FP64): off-diagonal
+  // blocks only (the product takes w_j - w_r), and the element records.
+  void* val[2] = {nullptr, nullptr};
+  void* elem[2] = {nullptr, nullptr};
 };
 
 // The vertex order and index arrays of the matrix, as the kernels take them.
@@ -69,10 +74,25 @@ __host__ __device__ inline int first_slice(int b, int grid, int nslice) {
 // EBB_OK with rm.state == -1: a vertex has more than kRowMaxTets tets, or the
 // memory does not suffice; the caller then keeps to the matrix-free maps.
 ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t stream);
-// Element records of K(u) and, with `force`, the element forces: u in planes
-// (stride nv) or interleaved 4-float elements (aos).
+// Element records of K(u) and, with `force` (FP64 only), the element forces:
+// u in planes (stride nv) or interleaved 4-float elements (aos).
 template <typename T>
 cudaError_t launch_element_blocks(ebb_rel_s* rel, int model, T mu0, T lam0, const T* u, bool aos, bool force, T* elem,
                                   cudaStream_t st);
+
+// Off-diagonal blocks of scale * K, zero on the rows of pinned vertices (pin may
+// be null; pin_bytes 1 or 4), from the element records.
+template <typename T>
+cudaError_t launch_row_blocks(const RowMatrix& m, const T* elem, const void* pin, int pin_bytes, T scale, T* val,
+                              cudaStream_t st);
+
+// Assembled K(u) on the rows and y += K w; *done is false when the rows do not
+// apply to the relation (or, for the product, hold no K in this precision).
+template <typename T>
+cudaError_t launch_row_assemble(ebb_rel_s* rel, int model, T mu0, T lam0, const MapIO<T>& io, cudaStream_t st,
+                                bool* done);
+template <typename T>
+cudaError_t launch_row_product(ebb_rel_s* rel, const T* w, T* y, bool aos, const int* active, cudaStream_t st,
+                               bool* done);
 
 }  // namespace ebb

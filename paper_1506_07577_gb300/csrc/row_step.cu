@@ -83,49 +83,6 @@ __global__ void row_mass_kernel(int nv, const int* __restrict__ off, const int* 
   m[v] = 0.25 * rho * s;
 }
 
-// One warp per slot: the off-diagonal blocks of dt^2 K, each the sum of its
-// contributions in increasing tet order; zero on pinned rows, so that a pinned
-// row's products stay zero.  FP64 adds and the latency of the record gathers
-// bound it about equally.
-constexpr int kBlockThreads = 256;
-
-template <typename PT>
-__global__ void __launch_bounds__(kBlockThreads)
-row_block_kernel(RowView m, int64_t nslots, const int* __restrict__ slot_slice, const int2* __restrict__ crange,
-                 const int* __restrict__ contrib, const double* __restrict__ elem, const PT* __restrict__ pin,
-                 double dt2, double* __restrict__ val, unsigned* bar) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *bar = 0u;   // the solve's barrier counter
-  const int64_t q = ((int64_t)blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (q >= nslots) return;
-  const int s = slot_slice[q];
-  const bool own = lane < 3 * kSliceRows;
-  const int i = own ? lane / 3 : 0, c = own ? lane - 3 * i : 0;
-  const int2 r = own ? crange[q * kSliceRows + i] : make_int2(0, 0);
-  const int v = own ? m.row_of[s * kSliceRows + i] : -1;
-  if (q == m.slice_off[s]) return;   // the diagonal blocks: formed by the solve
-  double x[3] = {0.0, 0.0, 0.0};
-  if (r.x < r.y && !pinned_at(pin, v)) {
-    auto rec_of = [&](int code, int& st) {
-      const bool tr = (code & 1) != 0;
-      st = tr ? 3 : 1;
-      return elem + (size_t)(code >> 4) * kElemLen + 9 * ((code >> 1) & 7) + (tr ? c : 3 * c);
-    };
-    int st;
-    const double* rec = rec_of(contrib[r.x], st);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) x[d] = rec[d * st];
-#pragma unroll 4
-    for (int e = r.x + 1; e < r.y; ++e) {
-      rec = rec_of(contrib[e], st);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) x[d] += rec[d * st];
-    }
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) val[((size_t)q * 3 + d) * 32 + lane] = dt2 * x[d];
-}
-
 // ---- the solve --------------------------------------------------------------
 enum RowFinish { FIN_STEP = 0, FIN_VELOCITY = 1, FIN_ADJOINT = 2 };
 
@@ -367,11 +324,11 @@ __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __
 #pragma unroll 2
         for (int e = a.voff[v] + k0; e < e1; e += kstep) {
           const int code = a.vent[e], corner = code & 3;
-          const double* rec = a.elem + (size_t)(code >> 2) * kElemLen + kElemForce + c;
+          const double* rec = a.elem + (size_t)(code >> 2) * kElemLen + 4 * c + 3;
           if (corner == 0)
-            f -= rec[0] + rec[3] + rec[6];
+            f -= rec[0] + rec[12] + rec[24];
           else
-            f += rec[3 * (corner - 1)];
+            f += rec[12 * (corner - 1)];
         }
       }
 #pragma unroll
@@ -640,10 +597,9 @@ ebb_status_t row_step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v
   RowCgArgs ca;
   memset(&ca, 0, sizeof ca);
   ca.m = RowView{m.nslice, m.slice_off, m.row_of, m.col};
-  const int64_t blocks = (m.nslots * 32 + kBlockThreads - 1) / kBlockThreads;
-  row_block_kernel<PT><<<(unsigned)std::max<int64_t>(1, blocks), kBlockThreads, 0, st>>>(
-      ca.m, m.nslots, m.slot_slice, m.crange, m.contrib, s->elem, pin, prm->dt * prm->dt, s->val, s->bar);
-  e = cudaGetLastError();
+  e = cudaMemsetAsync(s->bar, 0, sizeof(unsigned), st);
+  if (e == cudaSuccess)
+    e = launch_row_blocks<double>(m, s->elem, pin, (int)sizeof(PT), prm->dt * prm->dt, s->val, st);
   if (e != cudaSuccess) return cuda_check(ctx, e, "rows of the step matrix");
   ca.nv = nv;
   ca.val = s->val;
@@ -759,12 +715,12 @@ ebb_status_t row_step_ready(ebb_ctx_s* ctx, ebb_rel_s* tets, bool* yes) {
   *yes = false;
   ebb_status_t s = ensure_row_pattern(ctx, tets, ctx->stream);
   if (s) return s;
-  if (tets->rows->state != 1) return EBB_OK;
+  if (tets->rows->state != 1 || tets->rows->no_step) return EBB_OK;
   bool fits = false;
   s = ensure_row_step(ctx, tets, &fits);
   if (s) return s;
   if (!fits) {
-    tets->rows->state = -1;   // no room: the matrix-free step from now on
+    tets->rows->no_step = true;   // no room: the matrix-free step from now on
     return EBB_OK;
   }
   *yes = true;
