@@ -153,8 +153,11 @@ struct EdgeIndex {
   int* tet_blk = nullptr;
   void* blocks[2] = {nullptr, nullptr};
   bool assembled[2] = {false, false};
-  // Spring-mass system on the edges: rest length per entry (the self-loop's
-  // unused), double-buffered positions, energy partial sums.
+  // Spring-mass system on the edges: the springs in slices of 32 rows (slot
+  // layout in springs.cu) -- rows and their places, slot offsets, other ends,
+  // rest lengths -- a run's positions and velocities, energy partial sums.
+  int spring_slices = 0;
+  int *spring_row = nullptr, *spring_place = nullptr, *spring_off = nullptr, *spring_end = nullptr;
   void* rest[2] = {nullptr, nullptr};
   void* qbuf[2] = {nullptr, nullptr};
   double* epart = nullptr;

@@ -305,6 +305,10 @@ void free_edges(ebb_rel_s* tets) {
     cudaFree(E.qbuf[p]);
   }
   cudaFree(E.epart);
+  cudaFree(E.spring_row);
+  cudaFree(E.spring_place);
+  cudaFree(E.spring_off);
+  cudaFree(E.spring_end);
   E = EdgeIndex();
 }
 

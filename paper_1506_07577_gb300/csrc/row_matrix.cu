@@ -674,6 +674,11 @@ template cudaError_t launch_row_product<double>(ebb_rel_s*, const double*, doubl
 template cudaError_t launch_element_blocks<double>(ebb_rel_s*, int, double, double, const double*, bool, bool, double*,
                                                    cudaStream_t);
 
+cudaError_t exclusive_scan(int n, const int* in, int* out, cudaStream_t st) {
+  scan_kernel<<<1, kScanThreads, 0, st>>>(n, in, out);
+  return cudaGetLastError();
+}
+
 void free_row_matrix(ebb_rel_s* tets) {
   RowMatrix* m = tets->rows;
   if (!m) return;

@@ -74,6 +74,9 @@ __host__ __device__ inline int first_slice(int b, int grid, int nslice) {
 // EBB_OK with rm.state == -1: a vertex has more than kRowMaxTets tets, or the
 // memory does not suffice; the caller then keeps to the matrix-free maps.
 ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t stream);
+// Exclusive sums of n counts: out[0 .. n] (device arrays).
+cudaError_t exclusive_scan(int n, const int* in, int* out, cudaStream_t st);
+
 // Element records of K(u) and, with `force` (FP64 only), the element forces:
 // u in planes (stride nv) or interleaved 4-float elements (aos).
 template <typename T>
