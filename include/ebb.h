@@ -118,7 +118,9 @@ typedef enum { EBB_PREC_F64 = 0, EBB_PREC_F32 = 1 } ebb_precision_t;
  *           product and component r of every corner output, exchanging
  *           the rows it needs with its neighbours through warp shuffles;
  *           hardware atomic adds into the vertex fields.
- *   AUTO:   the autotuned choice (ebb_relation_autotune), else TILED. */
+ *   AUTO:   the autotuned choice (ebb_relation_autotune), else TILED in FP32
+ *           and for the host-buffer map, and in FP64 ATOMIC, or COOP on
+ *           relations of few tets (the FP64 pipe bounds FP64 maps). */
 typedef enum {
   EBB_REDUCE_ATOMIC = 0,
   EBB_REDUCE_COLOR = 1,
@@ -393,7 +395,7 @@ ebb_status_t ebb_map_tet_diagK(ebb_ctx_t ctx, ebb_rel_t tets, const char* u,
  * use the fastest tile size (the blobs are rebuilt if it changed) and
  * EBB_REDUCE_AUTO resolves to the fastest variant for this model and
  * precision in every map and step on the relation (before any autotune it
- * resolves to EBB_REDUCE_TILED).  Results are unaffected except for the
+ * resolves as EBB_REDUCE_AUTO says).  Results are unaffected except for the
  * order of floating-point additions.  Synchronous; allocates and frees an
  * output scratch field.  Errors: EBB_ERR_ARG / EBB_ERR_STATE as for the maps;
  * device errors of the timed maps (EBB_ERR_INVERTED) are returned. */
@@ -438,8 +440,8 @@ ebb_status_t ebb_relation_set_tuning(ebb_ctx_t ctx, ebb_rel_t tets, int32_t mode
  * side): how many tiles the tiled variants walk and how many tets each holds
  * at most, how many colours the coloured variant launches, whether FP32 tiled
  * maps stage their operands vertex-interleaved, whether vertices are
- * renumbered internally, and the variant EBB_REDUCE_AUTO resolves to per
- * [model][precision] (-1: not tuned, AUTO means TILED).  Errors:
+ * renumbered internally, and the autotuned variant of EBB_REDUCE_AUTO per
+ * [model][precision] (-1: not tuned).  Errors:
  * EBB_ERR_ARG (null argument), EBB_ERR_STATE (not finalized). */
 typedef struct {
   int64_t n_tets, n_verts;

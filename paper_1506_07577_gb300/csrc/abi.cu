@@ -194,15 +194,33 @@ bool valid_reduce(int r) {
          r == EBB_REDUCE_TILED_ORDERED || r == EBB_REDUCE_COOP;
 }
 
-// EBB_REDUCE_AUTO: the autotuned variant for this model and precision, else
-// the tiled one.
+constexpr int64_t kCoopTets = 8192;
+
+// EBB_REDUCE_AUTO: the autotuned variant for this model and precision, else by
+// precision and size.  FP32: the tiled one.  FP64 maps are bound by the FP64 pipe,
+// which the tiles' staging and reduction only add to: one thread per tet with
+// atomics from kCoopTets tets on, and below that three threads per tet, since
+// a warp's chain of FP64 instructions (64 cycles each) is then the map's time.
+// Measured, force and K w in us, tiled / atomic / three threads: StVK 2,560 tets
+// 18.5 / 16.4 / 10.3, 8,640 18.5 / 16.4 / 14.4, 40,000 41 / 37 / 40, 878,080
+// 567 / 481 / 731; neo-Hookean 8,640 20.5 / 18.5 / 18.5, 20,480 34 / 31 / 31.
 ebb_reduce_t resolve_reduce(const ebb_rel_s* tets, ebb_reduce_t r, int model, int precision) {
   if (r != EBB_REDUCE_AUTO) return r;
   if ((model == EBB_STVK || model == EBB_NEOHOOKEAN) && (precision == EBB_PREC_F64 || precision == EBB_PREC_F32)) {
     const int t = tets->tuned[model][precision];
     if (t >= 0) return (ebb_reduce_t)t;
   }
+  if (precision == EBB_PREC_F64) return tets->size < kCoopTets ? EBB_REDUCE_COOP : EBB_REDUCE_ATOMIC;
   return EBB_REDUCE_TILED;
+}
+
+// The same for the calls that work tile by tile: AUTO is the autotuned variant,
+// else the tiled one.
+ebb_reduce_t resolve_tiled(const ebb_rel_s* tets, ebb_reduce_t r, int model, int precision) {
+  const bool known = (model == EBB_STVK || model == EBB_NEOHOOKEAN) &&
+                     (precision == EBB_PREC_F64 || precision == EBB_PREC_F32);
+  if (r == EBB_REDUCE_AUTO && (!known || tets->tuned[model][precision] < 0)) return EBB_REDUCE_TILED;
+  return resolve_reduce(tets, r, model, precision);
 }
 
 // Resolve a vertex field used by a map or step; checks dtype and width.
@@ -252,7 +270,7 @@ ebb_status_t map_fields(ebb_ctx_s* ctx, ebb_rel_s* tets, const char* const* name
 // targets in every case.
 ebb_status_t launch_map_staged(ebb_ctx_s* ctx, ebb_rel_s* tets, int ops, int model, double mu, double lambda,
                                ebb_reduce_t reduce, bool f64, bool x4, void* const* in_user, int nin,
-                               void* const* out_user, int nout, bool drop) {
+                               void* const* out_user, int nout, bool drop, bool after_zero = false) {
   const int nv = (int)tets->verts->size;
   const size_t bytes = (size_t)nv * (x4 ? 16 : 3 * (f64 ? 8 : 4));
   // Reordered vertices are staged anyway, so their FP32 tiled maps always
@@ -296,8 +314,10 @@ ebb_status_t launch_map_staged(ebb_ctx_s* ctx, ebb_rel_s* tets, int ops, int mod
   }
   cudaError_t e;
   int oi = 0;
+  const bool beside = after_zero && !stage && !tets->vperm;   // nothing runs between the zeroing and the map
   if (f64) {
     MapIO<double> io;
+    io.after_zero = beside;
     io.u = (const double*)in[0];
     io.w = (const double*)in[1];
     if (ops & OP_FORCE) io.f = (double*)out[oi++];
@@ -308,6 +328,7 @@ ebb_status_t launch_map_staged(ebb_ctx_s* ctx, ebb_rel_s* tets, int ops, int mod
     tets->test_drop_tile = -1;
   } else {
     MapIO<float> io;
+    io.after_zero = beside;
     io.u = (const float*)in[0];
     io.w = (const float*)in[1];
     if (ops & OP_FORCE) io.f = (float*)out[oi++];
@@ -344,7 +365,9 @@ ebb_status_t run_map(ebb_ctx_t ctx, ebb_rel_t tets, const MapCall& mc, int ops, 
     return set_error(ctx, EBB_ERR_ARG, "unknown material model");
   if (opts->precision != EBB_PREC_F64 && opts->precision != EBB_PREC_F32)
     return set_error(ctx, EBB_ERR_ARG, "unknown precision");
-  const ebb_reduce_t reduce = resolve_reduce(tets, opts->reduce, opts->model, opts->precision);
+  const bool drop = (opts->flags & EBB_MAP_TEST_DROP_TILE) != 0;
+  const ebb_reduce_t reduce = drop ? resolve_tiled(tets, opts->reduce, opts->model, opts->precision)
+                                   : resolve_reduce(tets, opts->reduce, opts->model, opts->precision);
   if (!valid_reduce(reduce))
     return set_error(ctx, EBB_ERR_ARG, "unknown reduction variant");
   if (reduce == EBB_REDUCE_COLOR && !tets->has_colour)
@@ -375,17 +398,15 @@ ebb_status_t run_map(ebb_ctx_t ctx, ebb_rel_t tets, const MapCall& mc, int ops, 
       if (ranges_overlap(out[i], bytes, out[j], bytes))
         return set_error(ctx, EBB_ERR_PHASE, "two reduce targets of one map overlap");
   }
-  const bool drop = (opts->flags & EBB_MAP_TEST_DROP_TILE) != 0;
   if (drop && reduce != EBB_REDUCE_TILED)
     return set_error(ctx, EBB_ERR_ARG, "EBB_MAP_TEST_DROP_TILE needs the tiled reduction");
-  if (opts->flags & EBB_MAP_ZERO_OUT) {
-    for (int i = 0; i < mc.nout; ++i) {
-      ebb_status_t s = cuda_check(ctx, cudaMemsetAsync(out[i], 0, bytes, ctx->stream), "zeroing output");
-      if (s) return s;
-    }
+  const bool zero = (opts->flags & EBB_MAP_ZERO_OUT) != 0;
+  if (zero) {
+    ebb_status_t s = cuda_check(ctx, zero_fields(out, mc.nout, bytes, ctx->stream), "zeroing outputs");
+    if (s) return s;
   }
   return launch_map_staged(ctx, tets, ops, opts->model, opts->mu, opts->lambda, reduce, f64, x4, in, mc.nin, out,
-                           mc.nout, drop);
+                           mc.nout, drop, zero);
 }
 
 }  // namespace
@@ -1020,7 +1041,7 @@ ebb_status_t ebb_map_tet_force_Kv_host(ebb_ctx_t ctx, ebb_rel_t tets, const char
   }
   // The tiled map on fields it reads in place runs in chunks that overlap
   // the copies; every other form copies everything in, maps, copies out.
-  const ebb_reduce_t reduce = resolve_reduce(tets, opts->reduce, opts->model, opts->precision);
+  const ebb_reduce_t reduce = resolve_tiled(tets, opts->reduce, opts->model, opts->precision);
   const bool staged = !x4 && !f64 && tets->stage_interleaved;
   if (bytes > 0 && reduce == EBB_REDUCE_TILED && !tets->vperm && !staged &&
       !(opts->flags & EBB_MAP_TEST_DROP_TILE) && tets->tiles.ntiles >= 2 * HostPlan::kChunks) {

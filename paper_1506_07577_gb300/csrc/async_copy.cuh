@@ -11,6 +11,14 @@
 
 namespace ebb {
 
+// Programmatic dependent launch: wait until the kernels before this one have
+// finished and their writes are visible (returns at once when the kernel was
+// launched without that attribute), and let the next kernel's blocks start.
+__device__ __forceinline__ void wait_prior_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_next_kernel() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));
 }

@@ -14,6 +14,7 @@
 // its component of every corner output with one atomic.
 #pragma once
 
+#include "async_copy.cuh"
 #include "ebb_internal.h"
 #include "tet_io.cuh"
 #include "tet_math.cuh"
@@ -248,6 +249,7 @@ tet_coop_kernel(int nt, int nv, const int4* __restrict__ keys, const int* __rest
     }
     if (!good && act && r == 0) raise_error(err, EBB_ERR_INVERTED, perm[t]);
   }
+  wait_prior_kernel();
   if (!act || !good) return;
   // component r of every corner output, one atomic each
 #pragma unroll

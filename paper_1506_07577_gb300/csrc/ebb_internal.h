@@ -281,7 +281,14 @@ struct MapIO {
   // above is nv groups of 4 (x, y, z, padding) instead of 3 planes; FP32 and
   // the tiled reduction only.
   bool aos = false;
+  // The kernel before the map on the stream only zeroes the outputs: the map may
+  // start beside it and waits before it adds.
+  bool after_zero = false;
 };
+
+// Zero n (at most 3) buffers of `bytes` each (a multiple of 4, 4-byte aligned)
+// in one launch.
+cudaError_t zero_fields(void* const* p, int n, size_t bytes, cudaStream_t st);
 
 // Launch one element map over all tets of `rel` on `stream`.  `active`
 // (device int, may be null) lets the kernel return early when *active == 0

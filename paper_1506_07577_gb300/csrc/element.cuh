@@ -4,6 +4,7 @@
 
 #include "ebb_internal.h"
 #include "tet_math.cuh"
+#include "tet_math_f64.cuh"
 #include "tet_math_x2.cuh"
 
 namespace ebb {
@@ -33,6 +34,15 @@ __device__ __forceinline__ bool element_eval(const T* B, T V, T mu, T lam, const
         ko[a][c] = out[a][c].y;
       }
     return true;
+  }
+  if constexpr (sizeof(T) == 8 && (OPS & OP_DIAG) == 0) {
+    constexpr bool FO = (OPS & OP_FORCE) != 0, KV = (OPS & OP_KV) != 0;
+    if constexpr (MODEL == EBB_STVK) {
+      stvk_eval_f64<FO, KV>(B, V, mu, lam, Du, Dw, fo, ko);
+      return true;
+    } else {
+      return nh_eval_f64<FO, KV>(B, V, mu, lam, Du, Dw, fo, ko);
+    }
   }
   T G[9];
   mm(Du, B, G);

@@ -18,6 +18,7 @@
 // m |qd|^2 / 2 in FP64 in a fixed order.
 #include <algorithm>
 
+#include "async_copy.cuh"
 #include "ebb_internal.h"
 #include "row_matrix.cuh"
 
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(kStepThreads, sizeof(T) == 4 ? 8 : 4)
 spring_step_kernel(int nv, int nslice, const int* __restrict__ row_of, const int* __restrict__ slice_off,
                    const int* __restrict__ end, const T* __restrict__ rest, T k, T dt, const Quad<T>* __restrict__ qin,
                    Quad<T>* __restrict__ qout, Quad<T>* __restrict__ vel, T* q_planes, T* qd_planes) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  release_next_kernel();
   const int r = blockIdx.x * kStepThreads + threadIdx.x;
   const int s = r >> 5, lane = r & 31;
   const int v = s < nslice ? row_of[r] : -1;
@@ -153,7 +154,7 @@ spring_step_kernel(int nv, int nslice, const int* __restrict__ row_of, const int
   int h[kStepGroup];
 #pragma unroll
   for (int g = 0; g < kStepGroup; ++g) h[g] = g < nk ? ep[g * 32] : r;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  wait_prior_kernel();
   if (v < 0) return;
   const Quad<T> own = qin[r];
   const Quad<T> vi = vel[r];

@@ -20,7 +20,9 @@
 //           thread per vertex adds its rows in tile order (deterministic);
 //   gather  per-corner outputs to a buffer, then one thread per vertex sums
 //           its entries in index order (below).
+#include <algorithm>
 #include <cstdint>
+#include <utility>
 
 #include "async_copy.cuh"
 #include "coop.cuh"
@@ -34,6 +36,47 @@ namespace ebb {
 namespace {
 
 constexpr int kMapThreads = 128;
+
+// Launch `kernel`, beside the kernel before it on the stream when that one only
+// zeroes the outputs (the kernel waits for it before it adds).
+template <typename... P, typename... A>
+cudaError_t launch_after_zero(bool after_zero, void (*kernel)(P...), int grid, int threads, size_t smem,
+                              cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = after_zero ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+// ---- zeroing of the += targets (EBB_MAP_ZERO_OUT) ----------------------------
+// All outputs of a map in one launch (a launch each is 2 us, much of a small
+// map's time); 16-byte stores between the aligned bounds of each buffer.
+constexpr int kZeroThreads = 256;
+
+struct ZeroArgs {
+  char* p[3];
+  size_t bytes;
+};
+
+__global__ void __launch_bounds__(kZeroThreads) zero_kernel(ZeroArgs a) {
+  release_next_kernel();
+  char* p = a.p[blockIdx.y];
+  const size_t i = (size_t)blockIdx.x * kZeroThreads + threadIdx.x, n = (size_t)gridDim.x * kZeroThreads;
+  size_t head = (16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15;   // bytes before the first 16-byte bound
+  if (head > a.bytes) head = a.bytes;
+  const size_t quads = (a.bytes - head) / 16, tail = head + 16 * quads;
+  int4* q = reinterpret_cast<int4*>(p + head);
+  for (size_t k = i; k < quads; k += n) q[k] = make_int4(0, 0, 0, 0);
+  for (size_t b = 4 * i; b < head; b += 4 * n) *reinterpret_cast<int*>(p + b) = 0;
+  for (size_t b = tail + 4 * i; b < a.bytes; b += 4 * n) *reinterpret_cast<int*>(p + b) = 0;
+}
 
 // ---- direct: one thread per tet -------------------------------------------
 // AOS: vertex-interleaved operands (MapIO::aos, FP32): one 16-byte load per
@@ -55,8 +98,10 @@ tet_map_kernel(int t_begin, int t_end, int nt, int nv, const int4* __restrict__ 
   T fo[4][3], ko[4][3], dgo[4][3];
   if (!element_eval<T, MODEL, OPS>(B, V, mu, lam, Du, Dw, fo, ko, dgo)) {
     raise_error(err, EBB_ERR_INVERTED, perm[t]);
+    wait_prior_kernel();
     return;
   }
+  wait_prior_kernel();
   if constexpr (AOS) {
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
@@ -371,10 +416,10 @@ cudaError_t launch_tiles(ebb_rel_s* rel, T mu0, T lam0, const MapIO<T>& io, cons
   int grid = Cfg::grid_per_sm * sm_count();
   if (grid > count) grid = count;
   const int drop = rel->test_drop_tile;
-  tet_tile_kernel<T, MODEL, OPS, AOS, ORD><<<grid, kTileThreads, smem, stream>>>(
-      count, (int)rel->verts->size, blob_of<T>(tl) + (size_t)t0 * L.bytes, L, rel->tet_perm, mu0, lam0, io, active,
-      rel->ctx->d_err, drop, drop >= 0 ? kTestWaitCycles : kWaitCycles);
-  return cudaGetLastError();
+  return launch_after_zero(io.after_zero, tet_tile_kernel<T, MODEL, OPS, AOS, ORD>, grid, kTileThreads, smem, stream,
+                           count, (int)rel->verts->size, blob_of<T>(tl) + (size_t)t0 * L.bytes, L,
+                           (const int*)rel->tet_perm, mu0, lam0, io, active, rel->ctx->d_err, drop,
+                           drop >= 0 ? kTestWaitCycles : kWaitCycles);
 }
 
 // Partial rows of the ordered tiled variant (room for three outputs),
@@ -431,17 +476,16 @@ cudaError_t launch_range(int b, int e, int nt, int nv, const int4* keys, const i
   const int n = e - b;
   if (n <= 0) return cudaSuccess;
   const int grid = (n + kMapThreads - 1) / kMapThreads;
+  // one colour follows another: only the first launch may run beside the zeroing
+  const bool az = io.after_zero && ATOMIC;
   if (io.aos) {
-    if constexpr (sizeof(T) == 4) {
-      tet_map_kernel<T, MODEL, OPS, ATOMIC, true><<<grid, kMapThreads, 0, stream>>>(b, e, nt, nv, keys, perm, s, mu0,
-                                                                                    lam0, io, active, err);
-      return cudaGetLastError();
-    }
+    if constexpr (sizeof(T) == 4)
+      return launch_after_zero(az, tet_map_kernel<T, MODEL, OPS, ATOMIC, true>, grid, kMapThreads, 0, stream, b, e, nt,
+                               nv, keys, perm, s, mu0, lam0, io, active, err);
     return cudaErrorInvalidValue;
   }
-  tet_map_kernel<T, MODEL, OPS, ATOMIC, false><<<grid, kMapThreads, 0, stream>>>(b, e, nt, nv, keys, perm, s, mu0,
-                                                                                 lam0, io, active, err);
-  return cudaGetLastError();
+  return launch_after_zero(az, tet_map_kernel<T, MODEL, OPS, ATOMIC, false>, grid, kMapThreads, 0, stream, b, e, nt, nv,
+                           keys, perm, s, mu0, lam0, io, active, err);
 }
 
 template <typename T>
@@ -505,15 +549,15 @@ cudaError_t launch_coop(ebb_rel_s* rel, T mu0, T lam0, const MapIO<T>& io, const
   const int grid = (nt + kCoopTetsPerBlock - 1) / kCoopTetsPerBlock;
   if (io.aos) {
     if constexpr (sizeof(T) == 4) {
-      tet_coop_kernel<T, MODEL, OPS, true><<<grid, kCoopThreads, 0, stream>>>(
-          nt, nv, rel->keys, rel->tet_perm, streams_of<T>(rel, false), mu0, lam0, io, active, rel->ctx->d_err);
-      return cudaGetLastError();
+      return launch_after_zero(io.after_zero, tet_coop_kernel<T, MODEL, OPS, true>, grid, kCoopThreads, 0, stream, nt,
+                               nv, (const int4*)rel->keys, (const int*)rel->tet_perm, streams_of<T>(rel, false), mu0,
+                               lam0, io, active, rel->ctx->d_err);
     }
     return cudaErrorInvalidValue;
   }
-  tet_coop_kernel<T, MODEL, OPS, false><<<grid, kCoopThreads, 0, stream>>>(
-      nt, nv, rel->keys, rel->tet_perm, streams_of<T>(rel, false), mu0, lam0, io, active, rel->ctx->d_err);
-  return cudaGetLastError();
+  return launch_after_zero(io.after_zero, tet_coop_kernel<T, MODEL, OPS, false>, grid, kCoopThreads, 0, stream, nt, nv,
+                           (const int4*)rel->keys, (const int*)rel->tet_perm, streams_of<T>(rel, false), mu0, lam0, io,
+                           active, rel->ctx->d_err);
 }
 
 template <typename T, int MODEL, int OPS>
@@ -576,6 +620,17 @@ cudaError_t dispatch_ops(ebb_rel_s* rel, int ops, ebb_reduce_t reduce, T mu0, T 
 }
 
 }  // namespace
+
+cudaError_t zero_fields(void* const* p, int n, size_t bytes, cudaStream_t st) {
+  if (n <= 0 || bytes == 0) return cudaSuccess;
+  ZeroArgs a = {};
+  for (int i = 0; i < n; ++i) a.p[i] = static_cast<char*>(p[i]);
+  a.bytes = bytes;
+  const size_t blocks = (bytes / 16 + kZeroThreads - 1) / kZeroThreads;
+  const dim3 grid((unsigned)std::min<size_t>(std::max<size_t>(blocks, 1), 1216), (unsigned)n);
+  zero_kernel<<<grid, kZeroThreads, 0, st>>>(a);
+  return cudaGetLastError();
+}
 
 // Opt the tiled kernels into their dynamic shared-memory sizes on the current
 // device (done at finalize, never inside a stream capture).

@@ -387,6 +387,8 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
       return false;
     }
     if (tid == 0) mbar_arrive(&empty_v[sv]);
+    // Nothing has been added yet: from here on the outputs must be zeroed.
+    if (j == 0) wait_prior_kernel();
 
     // Phase 2: one reduction unit per thread: kUnitEntries independent loads.
     if constexpr (sizeof(T) == 4 && NF == 2) {
