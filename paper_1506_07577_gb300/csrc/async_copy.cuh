@@ -139,17 +139,17 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Named barrier 1 over the first `nthreads` threads, OR-reducing `v`.
+// Named barrier `bar` over NTHREADS threads, OR-reducing `v`.
 template <int NTHREADS>
-__device__ __forceinline__ bool named_sync_or(bool v) {
+__device__ __forceinline__ bool named_sync_or(int bar, bool v) {
   unsigned r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, 1, %2, q;\n\t"
+      "bar.red.or.pred p, %3, %2, q;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(r)
-      : "r"((unsigned)v), "n"(NTHREADS)
+      : "r"((unsigned)v), "n"(NTHREADS), "r"(bar)
       : "memory");
   return r != 0;
 }

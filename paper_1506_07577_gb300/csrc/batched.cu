@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "ebb_internal.h"
+#include "mixed_cg.h"
 
 namespace ebb {
 namespace {
@@ -324,6 +325,10 @@ struct BatchScratch {
   cudaEvent_t ev = nullptr;
   cudaGraphExec_t chunk = nullptr;
   std::vector<unsigned char> key;
+  std::vector<int> vstart;           // first vertex of each mesh, and nv
+  MixedPlan* mixed = nullptr;        // one-launch FP32 solve (mixed_cg.cu), its second
+  double* p2 = nullptr;              // direction array and host results
+  std::vector<MixedResult> h_res;
 };
 
 void free_batch_scratch(ebb_rel_s* rel) {
@@ -342,6 +347,8 @@ void free_batch_scratch(ebb_rel_s* rel) {
   cudaFree(s->part);
   cudaFree(s->sc);
   cudaFree(s->n_active);
+  cudaFree(s->p2);
+  free_mixed_plan(s->mixed);
   if (s->chunk) cudaGraphExecDestroy(s->chunk);
   if (s->ev) cudaEventDestroy(s->ev);
   if (s->stream) cudaStreamDestroy(s->stream);
@@ -392,6 +399,7 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   s->nv = nv;
   s->nmesh = nmesh;
   s->batch_ptr = batch;
+  s->vstart = vstart;
   const size_t n = (size_t)3 * nv;
   e = cudaMalloc(&s->table, sizeof(int) * (3 * (size_t)nb + 2 * (size_t)nmesh));
   for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaMalloc(&s->acc[i], n * sizeof(double));
@@ -499,6 +507,21 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
   kio.w = mixed ? pe : (const T*)s->p;
   kio.Kw = acc_kp;
   kio.aos = aos;
+  // FP32 steps with the tiled reduction solve in one launch.
+  bool one_launch = false;
+  if constexpr (sizeof(T) == 4) {
+    one_launch = prm->reduce == EBB_REDUCE_TILED && mixed_cg_ready(ctx, tets, s->vstart, &s->mixed);
+    if (one_launch && s->p2 == nullptr && cudaMalloc(&s->p2, (size_t)n * sizeof(double)) != cudaSuccess) {
+      s->p2 = nullptr;
+      cudaGetLastError();
+      one_launch = false;
+    }
+    if (one_launch) {
+      const MixedVectors mv{ue, pin, 1, s->mass, s->dinv, s->r, s->p, s->p2, s->y, s->qz, pe, acc_kp};
+      e = launch_mixed_cg(tets, s->mixed, prm->model, mu0, lam0, mv, prm->dt, prm->rtol, prm->max_iters, st);
+      if (e != cudaSuccess) return cuda_check(ctx, e, "batched CG solve");
+    }
+  }
   // Capture kChunk iterations once; re-capture when anything baked in changes.
   std::vector<unsigned char> key(sizeof(BatchConst) + 5 * sizeof(double) + 3 * sizeof(void*));
   {
@@ -512,7 +535,7 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
     const void* kp[3] = {pin, kio.u, kio.w};
     memcpy(k, kp, sizeof kp);
   }
-  if (!s->chunk || s->key != key) {
+  if (!one_launch && (!s->chunk || s->key != key)) {
     if (s->chunk) cudaGraphExecDestroy(s->chunk);
     s->chunk = nullptr;
     e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
@@ -551,7 +574,7 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
     s->key = key;
   }
   int launched = 0;
-  while (true) {
+  while (!one_launch) {
     int h_active = 0;
     e = cudaGraphLaunch(s->chunk, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h_active, s->n_active, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -563,14 +586,18 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
   }
   batch_finish_kernel<<<4 * 152, 256, 0, st>>>(n, prm->dt, s->y, u, v);
   e = cudaGetLastError();
+  s->h_res.resize(nmesh);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(s->h_sc.data(), s->sc, (size_t)nmesh * sizeof(MeshCg), cudaMemcpyDeviceToHost, st);
+    e = one_launch ? cudaMemcpyAsync(s->h_res.data(), mixed_results(s->mixed), (size_t)nmesh * sizeof(MixedResult),
+                                     cudaMemcpyDeviceToHost, st)
+                   : cudaMemcpyAsync(s->h_sc.data(), s->sc, (size_t)nmesh * sizeof(MeshCg), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_err, ctx->d_err, ERRW_WORDS * sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_check(ctx, e, "batched step finish");
   ebb_status_t status = EBB_OK;
   for (int m = 0; m < nmesh; ++m) {
-    const MeshCg& h = s->h_sc[m];
+    const MixedResult h = one_launch ? s->h_res[m]
+                                     : MixedResult{s->h_sc[m].rr, s->h_sc[m].bb, s->h_sc[m].iter, s->h_sc[m].status};
     const double rel = h.bb > 0.0 ? std::sqrt(h.rr / h.bb) : 0.0;
     ebb_status_t ms = h.status;
     if (ms == EBB_OK && prm->fail_on_max_iters && h.iter >= prm->max_iters && rel > prm->rtol)
@@ -584,7 +611,9 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
       status = ms;
       char buf[128];
       snprintf(buf, sizeof buf, "batch %d: %s", m,
-               ms == EBB_ERR_CG_BREAKDOWN ? "PCG breakdown" : "PCG not converged");
+               ms == EBB_ERR_CG_BREAKDOWN ? "PCG breakdown"
+               : ms == EBB_ERR_TIMEOUT    ? "a bounded device wait gave up"
+                                          : "PCG not converged");
       set_error(ctx, ms, buf);
     }
   }

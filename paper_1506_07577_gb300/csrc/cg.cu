@@ -23,6 +23,7 @@
 #include <string>
 
 #include "ebb_internal.h"
+#include "mixed_cg.h"
 
 namespace ebb {
 
@@ -577,6 +578,8 @@ struct StepScratch {
   double *vjp_w = nullptr, *vjp_kl = nullptr, *vjp_xq = nullptr;   // adjoint-only buffers
   double *u_int = nullptr, *v_int = nullptr;                        // state in the internal vertex order
   unsigned char* pin_int = nullptr;
+  MixedPlan* mixed = nullptr;   // one-launch FP32 solve (mixed_cg.cu), and its second direction array
+  double* p2 = nullptr;
 };
 
 void free_step_scratch(ebb_rel_s* rel) {
@@ -600,6 +603,8 @@ void free_step_scratch(ebb_rel_s* rel) {
   cudaFree(s->u_int);
   cudaFree(s->v_int);
   cudaFree(s->pin_int);
+  cudaFree(s->p2);
+  free_mixed_plan(s->mixed);
   if (s->chunk) cudaGraphExecDestroy(s->chunk);
   if (s->ev) cudaEventDestroy(s->ev);
   if (s->stream) cudaStreamDestroy(s->stream);
@@ -737,6 +742,18 @@ ebb_status_t step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, co
   kio.Kw = acc_kp;
   kio.aos = aos;
 
+  // FP32 steps with the tiled reduction solve in one launch; the others in
+  // captured chunks of iterations.
+  bool one_launch = false;
+  if constexpr (sizeof(T) == 4) {
+    one_launch = prm->reduce == EBB_REDUCE_TILED && !assembled && mixed_cg_ready(ctx, tets, {0, nv}, &s->mixed);
+    if (one_launch && s->p2 == nullptr && cudaMalloc(&s->p2, (size_t)n * sizeof(double)) != cudaSuccess) {
+      s->p2 = nullptr;
+      cudaGetLastError();
+      one_launch = false;
+    }
+  }
+
   // kChunk CG iterations (plus the status read-back) are captured once as a
   // CUDA graph and relaunched until the device reports convergence.
   ChunkKey key;
@@ -752,7 +769,7 @@ ebb_status_t step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, co
   key.c = c;
   key.pin = pin;
   key.u = kio.u;
-  if (!s->chunk || !s->have_key || memcmp(&key, &s->key, sizeof key) != 0) {
+  if (!one_launch && (!s->chunk || !s->have_key || memcmp(&key, &s->key, sizeof key) != 0)) {
     if (s->chunk) cudaGraphExecDestroy(s->chunk);
     s->chunk = nullptr;
     s->have_key = false;
@@ -809,10 +826,13 @@ ebb_status_t step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, co
     // replaces the forward solve.
     vel_diff_kernel<<<vgrid, 256, 0, st>>>(n, vjp->v_next, v, s->y);
     e = cudaGetLastError();
-  } else {
+  } else if (!one_launch) {
     e = run_chunks();
+  } else if constexpr (sizeof(T) == 4) {
+    const MixedVectors mv{ue, pin, (int)sizeof(PT), s->mass, s->dinv, s->r, s->p, s->p2, s->y, s->qz, pe, acc_kp};
+    e = launch_mixed_cg(tets, s->mixed, prm->model, mu0, lam0, mv, prm->dt, prm->rtol, prm->max_iters, st);
   }
-  if (e != cudaSuccess) return cuda_check(ctx, e, "CG chunk");
+  if (e != cudaSuccess) return cuda_check(ctx, e, "CG solve");
 
   if (vjp != nullptr) {
     // Adjoint of the step just solved (FP64, StVK): v' = v + dv, then the
@@ -836,19 +856,27 @@ ebb_status_t step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, co
     step_finish_kernel<<<vgrid, 256, 0, st>>>(n, prm->dt, s->y, u, v);
   }
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(s->h_sc, s->sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, st);
+  static_assert(sizeof(MixedResult) <= sizeof(CgScalars), "one host buffer");
+  if (e == cudaSuccess)
+    e = one_launch ? cudaMemcpyAsync(s->h_sc, mixed_results(s->mixed), sizeof(MixedResult), cudaMemcpyDeviceToHost, st)
+                   : cudaMemcpyAsync(s->h_sc, s->sc, sizeof(CgScalars), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ctx->h_err, ctx->d_err, ERRW_WORDS * sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_check(ctx, e, "step finish");
-  const CgScalars& h = *s->h_sc;
+  MixedResult h;
+  if (one_launch) {
+    memcpy(&h, s->h_sc, sizeof h);
+    status = h.status;
+  } else {
+    h = MixedResult{s->h_sc->rr, s->h_sc->bb, s->h_sc->iter, s->h_sc->status};
+  }
   const double rel = h.bb > 0.0 ? std::sqrt(h.rr / h.bb) : 0.0;
   if (rep) {
     rep->iters = h.iter;
     rep->rel_residual = rel;
   }
   // Device-raised errors (inverted elements) take precedence.
-  cudaError_t ce = cudaMemcpyAsync(ctx->h_err, ctx->d_err, ERRW_WORDS * sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-  if (ce != cudaSuccess) return cuda_check(ctx, ce, "status read");
   if (ctx->h_err[ERRW_CODE] != 0) {
     const int code = ctx->h_err[ERRW_CODE], idx = ctx->h_err[ERRW_INDEX];
     cudaMemsetAsync(ctx->d_err, 0, ERRW_WORDS * sizeof(int), st);

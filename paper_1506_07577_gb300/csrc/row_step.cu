@@ -21,6 +21,7 @@
 #include <cstdio>
 #include <cstring>
 
+#include "grid_barrier.cuh"
 #include "row_matrix.cuh"
 
 namespace ebb {
@@ -53,7 +54,6 @@ namespace {
 constexpr int kPlainThreads = 768;   // row_cg_kernel, one CTA per SM
 constexpr int kSplitThreads = 128;   // its form for few slices
 constexpr int kMaxGrid = kRowMaxGrid;   // partial sums per set
-constexpr long long kGridWaitCycles = 2000000000LL;  // about 1 s at 2 GHz
 
 // Streaming load of a matrix value (read once per product: not kept in L1,
 // which the gathered vector entries use).
@@ -122,29 +122,6 @@ struct RowCgShared {
   int active, ok;
 };
 
-__device__ __forceinline__ void arrive_release(unsigned* bar) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-}
-// Wait until the counter has reached `target` (which may have wrapped);
-// false after about a second.
-__device__ __forceinline__ bool wait_acquire(const unsigned* bar, unsigned target) {
-  const long long t0 = clock64();
-  while (true) {
-    unsigned n;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(bar) : "memory");
-    if ((int)(n - target) >= 0) return true;
-    if (clock64() - t0 > kGridWaitCycles) return false;
-  }
-}
-
-// Barrier over the grid in two halves, so that work no other block waits for
-// can run in between.  The counter only grows: round r is complete at
-// r * gridDim.x arrivals.
-__device__ __forceinline__ void grid_arrive(unsigned* bar, unsigned& round) {
-  ++round;
-  __syncthreads();
-  if (threadIdx.x == 0) arrive_release(bar);
-}
 template <int NP>
 __device__ __forceinline__ bool grid_join(RowCgShared<NP>& sh, const unsigned* bar, unsigned round) {
   if (threadIdx.x == 0) sh.ok = wait_acquire(bar, round * gridDim.x);

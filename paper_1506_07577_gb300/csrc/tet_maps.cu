@@ -314,7 +314,7 @@ tet_tile_kernel(int ntiles, int nv, const unsigned char* __restrict__ blobs, Blo
   const int G = gridDim.x;
   if ((int)blockIdx.x >= ntiles) return;
   const int n_my = (ntiles - (int)blockIdx.x + G - 1) / G;
-  const TileView<T, OPS> V = tile_view<T, OPS>(smem, L);
+  const TileView<T, OPS> V = tile_view<T, OPS>(smem, L, threadIdx.x, blockIdx.x, G, 1);
   tile_init(V);
   __syncthreads();
   tile_map_pass<T, MODEL, OPS, AOS, ORD>(V, n_my, 0, nv, blobs, L, perm, mu0, lam0, io, err, drop_tile, wait_cycles);

@@ -124,12 +124,21 @@ struct TileView {
   uint64_t* full_v;
   uint64_t* empty_v;
   volatile int* abort_flag;
+  // Which walker of the tiles this is: thread within it, its number and how
+  // many there are (walker w maps tiles w, w + n, ...), and its named barrier.  A
+  // map kernel's CTA is one walker; a kernel may also hold several per CTA.
+  int tid, walker, nwalkers, bar;
 };
 
 template <typename T, int OPS>
-__device__ __forceinline__ TileView<T, OPS> tile_view(unsigned char* smem, const BlobLayout& L) {
+__device__ __forceinline__ TileView<T, OPS> tile_view(unsigned char* smem, const BlobLayout& L, int tid, int walker,
+                                                      int nwalkers, int bar) {
   using Z = TileSmem<T, OPS>;
   TileView<T, OPS> v;
+  v.tid = tid;
+  v.walker = walker;
+  v.nwalkers = nwalkers;
+  v.bar = bar;
   v.ring = smem;
   v.slots = reinterpret_cast<T*>(smem + Z::slot_off(L));
   v.outs = reinterpret_cast<T*>(smem + Z::out_off(L));
@@ -141,11 +150,11 @@ __device__ __forceinline__ TileView<T, OPS> tile_view(unsigned char* smem, const
   return v;
 }
 
-// Barrier initialisation by thread 0 (the caller then syncs the CTA).
+// Barrier initialisation by the walker's thread 0 (the caller then syncs the CTA).
 template <typename T, int OPS>
 __device__ __forceinline__ void tile_init(const TileView<T, OPS>& V) {
   using Z = TileSmem<T, OPS>;
-  if (threadIdx.x == 0) {
+  if (V.tid == 0) {
 #pragma unroll
     for (int r = 0; r < Z::RB; ++r) {
       mbar_init(&V.full_b[r], 1);
@@ -161,8 +170,7 @@ __device__ __forceinline__ void tile_init(const TileView<T, OPS>& V) {
   }
 }
 
-// One pass of the map over this CTA's tiles blockIdx.x, blockIdx.x + G, ...
-// (n_my of them).  `jbase` counts the tiles this CTA went through in earlier
+// One pass of the map over this walker's tiles (n_my of them).  `jbase` counts the tiles this CTA went through in earlier
 // passes over the same rings, so that ring stages and barrier phases carry
 // on from one pass to the next.  Returns false in a thread that gave up waiting or saw the
 // abort flag (the timeout is raised in `err`; the producer has drained its
@@ -181,11 +189,19 @@ __device__ __forceinline__ void st_part4(double* p, double x, double y, double z
   reinterpret_cast<double2*>(p)[1] = make_double2(z, 0.0);
 }
 
-template <typename T, int MODEL, int OPS, bool AOS, bool ORD>
+// `gate` is asked by the producer before its first gather, when its first blob
+// copies are on their way: it waits until the vertex fields may be read (and
+// returns false if it gave up).
+struct OpenGate {
+  __device__ __forceinline__ bool operator()() const { return true; }
+};
+
+template <typename T, int MODEL, int OPS, bool AOS, bool ORD, typename Gate = OpenGate>
 __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_my, int jbase, int nv,
                                               const unsigned char* __restrict__ blobs, const BlobLayout& L,
                                               const int* __restrict__ perm, T mu0, T lam0, const MapIO<T>& io,
-                                              int* err, int drop_tile, long long wait_cycles) {
+                                              int* err, int drop_tile, long long wait_cycles,
+                                              const Gate& gate = Gate()) {
   using Z = TileSmem<T, OPS>;
   constexpr int TT = Z::TT, NF = Z::NF, RB = Z::RB, RV = Z::RV;
   unsigned char* ring = V.ring;
@@ -196,9 +212,9 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
   uint64_t* full_v = V.full_v;
   uint64_t* empty_v = V.empty_v;
   volatile int* abort_flag = V.abort_flag;
-  const int tid = threadIdx.x;
+  const int tid = V.tid;
   const int lane = tid & 31;
-  const int G = gridDim.x;
+  const int G = V.nwalkers;
 
   if (tid >= TT) {
     // ---------------------------------------------------------- producer --
@@ -213,7 +229,7 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
           bad = true;
           break;
         }
-        const int tj = (int)blockIdx.x + j * G;
+        const int tj = V.walker + j * G;
         if (tj != drop_tile) {  // drop_tile: failure-detection tests only (-1 otherwise)
           if (lane == 0) {
             // Blobs are read once per map: evict them first, so that the
@@ -232,6 +248,7 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
         const int sb = JJ % RB, sv = JJ % RV;
         bool ok = mbar_wait_or_abort(&full_b[sb], (JJ / RB) & 1u, abort_flag, wait_cycles);
         if (ok) pend &= ~(1u << sb);
+        if (jj == 0) ok = gate() && ok;
         ok = ok && (JJ < RV || mbar_wait_or_abort(&empty_v[sv], ((JJ / RV) - 1) & 1u, abort_flag, wait_cycles));
         if (__any_sync(0xffffffffu, !ok)) {
           bad = true;
@@ -265,7 +282,7 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
     cp_async_wait_all();
     if (bad) {
       if (lane == 0) {
-        raise_error(err, EBB_ERR_TIMEOUT, blockIdx.x);
+        raise_error(err, EBB_ERR_TIMEOUT, V.walker);
         *abort_flag = 1;
       }
       // Bounded drain of the bulk copies still in flight before the CTA's
@@ -294,7 +311,7 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
     // ordered variant: this unit's partial row, loaded now and used after
     // phase 1 (the tile index is absolute: the ordered map maps every tile)
     int urow = -1;
-    if constexpr (ORD) urow = __ldg(io.unit_row + ((size_t)blockIdx.x + (size_t)j * G) * TT + tid);
+    if constexpr (ORD) urow = __ldg(io.unit_row + ((size_t)V.walker + (size_t)j * G) * TT + tid);
     T* sob = outs + (Z::OB == 2 ? (J & 1) : 0) * Z::out_elems;
     const bool ok = mbar_wait_or_abort(&full_b[sb], (J / RB) & 1u, abort_flag, wait_cycles) &&
                     mbar_wait_or_abort(&full_v[sv], (J / RV) & 1u, abort_flag, wait_cycles);
@@ -364,7 +381,7 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
       if (!good) raise_error(err, EBB_ERR_INVERTED, perm[h.z + tid]);
     }
     // With one output buffer, the previous tile's phase 2 must be done with it.
-    if (Z::OB == 1) named_sync_or<TT>(false);
+    if (Z::OB == 1) named_sync_or<TT>(V.bar, false);
     if (tid < h.x) {
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
@@ -379,9 +396,9 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
         }
       }
     }
-    if (named_sync_or<TT>(!ok)) {
+    if (named_sync_or<TT>(V.bar, !ok)) {
       if (tid == 0) {
-        raise_error(err, EBB_ERR_TIMEOUT, blockIdx.x);
+        raise_error(err, EBB_ERR_TIMEOUT, V.walker);
         *abort_flag = 1;
       }
       return false;
