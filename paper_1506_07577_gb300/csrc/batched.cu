@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "ebb_internal.h"
+#include "fp64_lean.cuh"
 #include "mixed_cg.h"
 
 namespace ebb {
@@ -146,8 +147,8 @@ batch_init_kernel(BatchConst c, BatchTable tb, const unsigned char* __restrict__
       const size_t ie = eidx<AOS>(c.nv, v, comp);
       double b = 0.0, di = 1.0;
       if (!pinned) {
-        b = c.dt * ((double)acc_f[ie] + mv * c.g[comp] - c.dt * (double)acc_kv[ie]);
-        di = 1.0 / (mv + c.dt * c.dt * (double)acc_d[ie]);
+        b = c.dt * (to_f64(acc_f[ie]) + mv * c.g[comp] - c.dt * to_f64(acc_kv[ie]));
+        di = recip(mv + c.dt * c.dt * to_f64(acc_d[ie]));
       }
       const double z = b * di;
       r[i] = b;
@@ -276,14 +277,26 @@ template <typename T, bool AOS>
 __global__ void batch_prep_kernel(int nv, const double* __restrict__ u, const double* __restrict__ v, T* ue, T* ve,
                                   T* acc_f, T* acc_kv, T* acc_d, T* acc_kp, bool copy) {
   for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nv; x += gridDim.x * blockDim.x) {
+    if constexpr (AOS) {
+      // whole 16-byte elements
+      const size_t n = nv;
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+      reinterpret_cast<float4*>(ue)[x] = make_float4(narrow(u[x]), narrow(u[n + x]), narrow(u[2 * n + x]), 0.f);
+      reinterpret_cast<float4*>(ve)[x] = make_float4(narrow(v[x]), narrow(v[n + x]), narrow(v[2 * n + x]), 0.f);
+      reinterpret_cast<float4*>(acc_f)[x] = zero;
+      reinterpret_cast<float4*>(acc_kv)[x] = zero;
+      reinterpret_cast<float4*>(acc_d)[x] = zero;
+      reinterpret_cast<float4*>(acc_kp)[x] = zero;
+    } else {
 #pragma unroll
-    for (int k = 0; k < (AOS ? 4 : 3); ++k) {
-      const size_t i = eidx<AOS>(nv, x, k);
-      if (copy) {
-        ue[i] = k < 3 ? (T)u[(size_t)k * nv + x] : T(0);
-        ve[i] = k < 3 ? (T)v[(size_t)k * nv + x] : T(0);
+      for (int k = 0; k < 3; ++k) {
+        const size_t i = eidx<AOS>(nv, x, k);
+        if (copy) {
+          ue[i] = (T)u[i];
+          ve[i] = (T)v[i];
+        }
+        acc_f[i] = acc_kv[i] = acc_d[i] = acc_kp[i] = T(0);
       }
-      acc_f[i] = acc_kv[i] = acc_d[i] = acc_kp[i] = T(0);
     }
   }
 }

@@ -281,6 +281,11 @@ struct MapIO {
   // above is nv groups of 4 (x, y, z, padding) instead of 3 planes; FP32 and
   // the tiled reduction only.
   bool aos = false;
+  // K w alone on interleaved operands, tiled: add only into the vertices v_lo ..
+  // v_lo + v_span - 1 (a batch solved in groups of meshes, whose border tiles
+  // hold tets of both neighbours).
+  int v_lo = 0;
+  unsigned v_span = 0xffffffffu;
   // The kernel before the map on the stream only zeroes the outputs: the map may
   // start beside it and waits before it adds.
   bool after_zero = false;

@@ -17,12 +17,18 @@
 // can be late.  At (b) the walkers' first tile copies are already on their way:
 // the producers wait there themselves.  The arithmetic is the separate kernels'.
 //
+// A batch is solved as two groups of meshes by two such kernels at once, each with
+// two walkers per SM: nothing ties them together, so that one group's vectors and
+// the other's maps share the SM.
+//
 // A block owns consecutive vertices, cut where a mesh ends into segments; a mesh's
 // dot products are the sums over its segments in order, formed alike in every
 // block that has one of them, so no scalars are exchanged.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 
+#include "fp64_lean.cuh"
 #include "grid_barrier.cuh"
 #include "mixed_cg.h"
 #include "tile_map.cuh"
@@ -42,33 +48,46 @@ struct MixedCg {
   int iter, status;
 };
 
-struct MixedPlan {
-  int nmesh = 0, nseg = 0, grid = 0;
-  std::vector<int> vstart;
-  void* slab = nullptr;
+// The part of a plan that one kernel solves.
+struct MixedGroup {
+  int v0 = 0, v1 = 0, tile0 = 0, tile1 = 0;
+  int nseg = 0;
   MixedSeg* seg = nullptr;
   int* first = nullptr;       // grid + 1: first segment of each block
   MixedCg* cg = nullptr;
   double* part = nullptr;     // 2 values x nseg, and 1 x nseg
-  MixedResult* res = nullptr;
   unsigned* ctl = nullptr;    // [0] barrier counter, [1] meshes that iterate
+};
+
+struct MixedPlan {
+  int ngroup = 0, grid = 0;
+  unsigned layout_gen = 0;    // the tiles the groups were cut from
+  MixedGroup group[2];
+  MixedResult* res = nullptr;
+  void* slab = nullptr;
+  cudaStream_t side = nullptr;   // the second group's stream
+  cudaEvent_t fork = nullptr, join = nullptr;
 };
 
 namespace {
 
-constexpr int kWalkers = 5;
-constexpr int kAuxWarps = 3;
-constexpr int kMapThreadsAll = kWalkers * kTileThreads;
-constexpr int kMixThreads = kMapThreadsAll + 32 * kAuxWarps;
-constexpr int kVecThreads = 768;                       // run the vector passes
-static_assert(kVecThreads <= kMapThreadsAll, "the vector passes' threads are walkers'");
-constexpr int kSegBatch = 8;    // segments whose sums are formed together
+// A block's shape: walkers, further warps, and how many threads run the vector
+// passes (a value's partials fit a walker's output rows).
+template <int WALKERS, int AUX, int VEC>
+struct Shape {
+  static constexpr int walkers = WALKERS, aux = AUX, vec = VEC;
+  static constexpr int map_threads = WALKERS * kTileThreads, threads = map_threads + 32 * AUX;
+};
+using One = Shape<5, 3, 768>;    // one block per SM
+using Half = Shape<2, 4, 448>;   // two blocks per SM, one of each group
+constexpr int kSegBatch = 6;    // segments whose sums are formed together
 constexpr int kCached = 4;      // segments of a block kept in shared memory
 using Tile = TileSmem<float, OP_KV>;
-static_assert(Tile::OB * Tile::out_elems * sizeof(float) >= kVecThreads * sizeof(double), "room for a value's partials");
+static_assert(Tile::OB * Tile::out_elems * sizeof(float) >= One::vec * sizeof(double), "room for a value's partials");
 
 struct MixedArgs {
-  int nv, ntiles;
+  int nv, ntiles, v_lo;
+  unsigned v_span;
   const unsigned char* blobs;
   BlobLayout L;
   const int* perm;
@@ -98,34 +117,8 @@ __device__ __forceinline__ double warp_sum(double x) {
   return x;
 }
 
-// An FP32 value in FP64, exactly, by integer instructions: a conversion costs as
-// much of the FP64 pipe as a multiplication.  Zero and normal values; the others
-// take the conversion.
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
-  if (m - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
-  if (m == 0u) return __hiloint2double((int)u, 0);
-  return (double)x;
-}
-
-// The FP32 value of x (round to nearest even), likewise: a conversion costs the
-// FP64 pipe as much.  Results in FP32's normal range and zero; the others
-// take the conversion.
-__device__ __forceinline__ float narrow(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned m = hi & 0x7fffffffu;
-  if (m - 0x38100000u < 0x0fd00000u) {   // 2^-126 <= |x| < 2^127
-    const unsigned t = ((m - 0x38000000u) << 3) | (lo >> 29), rest = lo << 3;   // kept bits, dropped bits
-    const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (t & 1u)) ? 1u : 0u;
-    return __uint_as_float((hi & 0x80000000u) | (t + up));
-  }
-  if ((m | lo) == 0u) return __uint_as_float(hi);
-  return (float)x;
-}
-
 struct MixedShared {
-  double* v[2];   // kVecThreads values each: the first two walkers' output rows, idle between maps
+  double* v[2];   // a value per vector thread each: the first two walkers' output rows, idle between maps
   double w[2][4];
   double tot[kSegBatch][2];
   MixedCg cg[kCached];
@@ -134,10 +127,10 @@ struct MixedShared {
 };
 
 // Partial sums of NV values of segment `s` (block-uniform) from every thread.
-template <int NV>
+template <int VEC, int NV>
 __device__ __forceinline__ void segment_partial(MixedShared& sh, const double (&x)[NV], double* part, int nseg, int s) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid < kVecThreads) {
+  if (tid < VEC) {
 #pragma unroll
     for (int j = 0; j < NV; ++j) sh.v[j][tid] = x[j];
   }
@@ -146,7 +139,8 @@ __device__ __forceinline__ void segment_partial(MixedShared& sh, const double (&
     const int j = warp >> 2, g = warp & 3, at = g * 32 + lane;
     double t = sh.v[j][at];
 #pragma unroll
-    for (int i = 1; i < kVecThreads / 128; ++i) t += sh.v[j][at + 128 * i];
+    for (int i = 1; i < (VEC + 127) / 128; ++i)
+      if (VEC % 128 == 0 || at + 128 * i < VEC) t += sh.v[j][at + 128 * i];
     t = warp_sum(t);
     if (lane == 0) sh.w[j][g] = t;
   }
@@ -198,8 +192,9 @@ struct IterationGate {
   __device__ __forceinline__ bool operator()() const { return wait_acquire(bar, target); }
 };
 
-template <int MODEL, typename PT>
-__global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
+template <typename SH, int MODEL, typename PT>
+__global__ void __launch_bounds__(SH::threads, SH::threads > 512 ? 1 : 2) mixed_cg_kernel(MixedArgs a) {
+  constexpr int kWalkers = SH::walkers, kVecThreads = SH::vec, kMixThreads = SH::threads;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ MixedShared sh;
   const int tid = threadIdx.x;
@@ -230,6 +225,8 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
   io.w = a.v.pe;
   io.Kw = a.v.acc;
   io.aos = true;
+  io.v_lo = a.v_lo;
+  io.v_span = a.v_span;
   __syncthreads();
 
   // r.z and r.r of the start
@@ -243,7 +240,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
         x[0] = fma(r, a.v.p[(size_t)k * nv + v], x[0]);
         x[1] = fma(r, r, x[1]);
       }
-    segment_partial<2>(sh, x, part2, a.nseg, s0 + s);
+    segment_partial<kVecThreads, 2>(sh, x, part2, a.nseg, s0 + s);
   }
   grid_arrive(bar, round);
   bool ok = grid_join(sh, bar, round);
@@ -304,7 +301,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
                           V, n_my, it * n_my, nv, a.blobs, a.L, a.perm, a.mu0, a.lam0, io, a.err, -1, kWaitCycles, gate))
         sh.bad = 1;
     } else if (it > 0) {
-      finish_y(pn, tid - kMapThreadsAll, 32 * kAuxWarps);
+      finish_y(pn, tid - SH::map_threads, 32 * SH::aux);
     }
     grid_arrive(bar, round);
     ok = grid_join(sh, bar, round) && sh.bad == 0;
@@ -330,7 +327,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
           x[0] = fma(pv[k], q, x[0]);
         }
       }
-      segment_partial<1>(sh, x, part1, a.nseg, s0 + s);
+      segment_partial<kVecThreads, 1>(sh, x, part1, a.nseg, s0 + s);
     }
     grid_arrive(bar, round);
     ok = grid_join(sh, bar, round);
@@ -376,7 +373,7 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
           x[1] = fma(ri, ri, x[1]);
         }
       }
-      segment_partial<2>(sh, x, part2, a.nseg, s0 + s);
+      segment_partial<kVecThreads, 2>(sh, x, part2, a.nseg, s0 + s);
     }
     grid_arrive(bar, round);
     ok = grid_join(sh, bar, round);
@@ -432,74 +429,90 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_cg_kernel(MixedArgs a) {
     }
 }
 
-template <int MODEL, typename PT>
+template <typename SH, int MODEL, typename PT>
 cudaError_t launch(const MixedArgs& a, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kMixThreads);
-  cfg.dynamicSmemBytes = kWalkers * a.walker_smem;
+  cfg.blockDim = dim3(SH::threads);
+  cfg.dynamicSmemBytes = SH::walkers * a.walker_smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, mixed_cg_kernel<MODEL, PT>, a);
+  return cudaLaunchKernelEx(&cfg, mixed_cg_kernel<SH, MODEL, PT>, a);
 }
 
 size_t walker_bytes(const BlobLayout& L) { return (Tile::bytes(L) + 127) / 128 * 128; }
 
-template <int MODEL, typename PT>
-bool resident(size_t smem) {
+// Do `want` blocks fit an SM?
+template <typename SH, int MODEL, typename PT>
+bool resident(size_t walker, int want) {
   int n = 0;
-  if (cudaFuncSetAttribute(mixed_cg_kernel<MODEL, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return false;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, mixed_cg_kernel<MODEL, PT>, kMixThreads, smem) ==
-             cudaSuccess &&
-         n >= 1;
+  const size_t smem = SH::walkers * walker;
+  auto* k = mixed_cg_kernel<SH, MODEL, PT>;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess) return false;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, SH::threads, smem) == cudaSuccess && n >= want;
 }
 
-}  // namespace
-
-void free_mixed_plan(MixedPlan* plan) {
-  if (!plan) return;
-  cudaFree(plan->slab);
-  delete plan;
+// First tile that holds a tet of vertices >= v (the tets of a batch are ordered
+// mesh by mesh), and whether it also holds a tet before; -1 when a copy fails.
+int border_tile(ebb_rel_s* rel, int v, bool* mixed) {
+  auto first_key = [&](int t, int* k) {
+    return cudaMemcpy(k, &rel->keys[t].x, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess;
+  };
+  int lo = 0, hi = (int)rel->size;
+  while (lo < hi) {
+    const int m = lo + (hi - lo) / 2;
+    int k = 0;
+    if (!first_key(m, &k)) return -1;
+    if (k < v)
+      lo = m + 1;
+    else
+      hi = m;
+  }
+  const int tet = lo;
+  *mixed = false;
+  if (tet >= (int)rel->size) return rel->tiles.ntiles;
+  auto first_tet = [&](int tile, int* z) {
+    int4 h;
+    if (cudaMemcpy(&h, rel->tiles.blob32 + (size_t)tile * rel->tiles.L32.bytes, sizeof h, cudaMemcpyDeviceToHost) !=
+        cudaSuccess)
+      return false;
+    *z = h.z;
+    return true;
+  };
+  lo = 0;
+  hi = rel->tiles.ntiles;   // the last tile whose first tet is <= tet
+  while (hi - lo > 1) {
+    const int m = (lo + hi) / 2;
+    int z = 0;
+    if (!first_tet(m, &z)) return -1;
+    if (z <= tet)
+      lo = m;
+    else
+      hi = m;
+  }
+  int z = 0;
+  if (!first_tet(lo, &z)) return -1;
+  *mixed = z < tet;
+  return lo;
 }
 
-const MixedResult* mixed_results(const MixedPlan* plan) { return plan->res; }
-
-bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vstart, MixedPlan** out) {
-  if (*out) return (*out)->grid > 0;
-  MixedPlan* m = new MixedPlan();
-  *out = m;   // grid 0: does not apply
-  const int nv = vstart.back(), nmesh = (int)vstart.size() - 1;
-  int nsm = 0;
-  if (rel->tiles.ntiles == 0 || nv == 0 ||
-      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || nsm < 1) {
-    cudaGetLastError();
-    return false;
-  }
-  // A block per SM: small meshes too, for whose few vertices and tiles more SMs
-  // mean shorter passes.
-  const int grid = nsm;
-  // Segments are summed one after the other: a batch of very many meshes is better
-  // off with a block per mesh.
-  if (nmesh > 16 * grid) return false;
-  const size_t smem = kWalkers * walker_bytes(rel->tiles.L32);
-  if (!resident<EBB_STVK, unsigned char>(smem) || !resident<EBB_NEOHOOKEAN, unsigned char>(smem) ||
-      !resident<EBB_STVK, int>(smem) || !resident<EBB_NEOHOOKEAN, int>(smem)) {
-    cudaGetLastError();
-    return false;
-  }
-  std::vector<MixedSeg> seg;
-  std::vector<int> first(grid + 1, 0), part0(nmesh + 1, 0);
-  int mesh = 0;
+// Segments of the vertices [v0, v1) over `grid` blocks; meshes numbered as in vstart.
+void cut_segments(const std::vector<int>& vstart, int v0, int v1, int grid, std::vector<MixedSeg>& seg,
+                  std::vector<int>& first) {
+  const int n = v1 - v0;
+  first.assign(grid + 1, 0);
+  std::vector<int> part0;   // first segment of each mesh met, in order
+  std::vector<int> meshes;
+  int mesh = (int)(std::upper_bound(vstart.begin(), vstart.end(), v0) - vstart.begin()) - 1;
   for (int b = 0; b < grid; ++b) {
     first[b] = (int)seg.size();
-    int v = (int)((long long)b * nv / grid);
-    const int end = (int)((long long)(b + 1) * nv / grid);
+    int v = v0 + (int)((long long)b * n / grid);
+    const int end = v0 + (int)((long long)(b + 1) * n / grid);
     while (v < end) {
       while (vstart[mesh + 1] <= v) ++mesh;
       const int e = std::min(end, vstart[mesh + 1]);
@@ -509,77 +522,180 @@ bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vsta
       s.v1 = e;
       s.lead = v == vstart[mesh] ? 1 : 0;
       s.part0 = s.npart = 0;
-      if (s.lead) part0[mesh] = (int)seg.size();
+      if (s.lead) {
+        part0.push_back((int)seg.size());
+        meshes.push_back(mesh);
+      }
       seg.push_back(s);
       v = e;
     }
   }
   first[grid] = (int)seg.size();
-  const int nseg = (int)seg.size();
-  part0[nmesh] = nseg;
+  part0.push_back((int)seg.size());
   for (MixedSeg& s : seg) {
-    s.part0 = part0[s.mesh];
-    s.npart = part0[s.mesh + 1] - part0[s.mesh];
+    const int k = s.mesh - meshes[0];
+    s.part0 = part0[k];
+    s.npart = part0[k + 1] - part0[k];
   }
+}
+
+}  // namespace
+
+void free_mixed_plan(MixedPlan* plan) {
+  if (!plan) return;
+  cudaFree(plan->slab);
+  if (plan->fork) cudaEventDestroy(plan->fork);
+  if (plan->join) cudaEventDestroy(plan->join);
+  if (plan->side) cudaStreamDestroy(plan->side);
+  delete plan;
+}
+
+const MixedResult* mixed_results(const MixedPlan* plan) { return plan->res; }
+
+bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vstart, MixedPlan** out) {
+  if (*out && (*out)->layout_gen != rel->layout_gen) {   // tiles cut again
+    free_mixed_plan(*out);
+    *out = nullptr;
+  }
+  if (*out) return (*out)->grid > 0;
+  MixedPlan* m = new MixedPlan();
+  *out = m;   // grid 0: does not apply
+  m->layout_gen = rel->layout_gen;
+  const int nv = vstart.back(), nmesh = (int)vstart.size() - 1;
+  int nsm = 0;
+  if (rel->tiles.ntiles == 0 || nv == 0 ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || nsm < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  // A block per SM and group: small meshes too, for whose few vertices and tiles
+  // more SMs mean shorter passes.
+  const int grid = nsm;
+  // Segments are summed one after the other: a batch of very many meshes is better
+  // off with a block per mesh.
+  if (nmesh > 16 * grid) return false;
+  const size_t walker = walker_bytes(rel->tiles.L32);
+  if (!resident<One, EBB_STVK, unsigned char>(walker, 1) || !resident<One, EBB_NEOHOOKEAN, unsigned char>(walker, 1) ||
+      !resident<One, EBB_STVK, int>(walker, 1) || !resident<One, EBB_NEOHOOKEAN, int>(walker, 1)) {
+    cudaGetLastError();
+    return false;
+  }
+  m->ngroup = 1;
+  m->group[0].v1 = nv;
+  m->group[0].tile1 = rel->tiles.ntiles;
+  // Two groups, cut between meshes nearest the middle vertex.
+  if (nmesh > 1 && resident<Half, EBB_STVK, unsigned char>(walker, 2) &&
+      resident<Half, EBB_NEOHOOKEAN, unsigned char>(walker, 2)) {
+    int cut = 1;
+    for (int k = 2; k < nmesh; ++k)
+      if (std::abs(2LL * vstart[k] - nv) < std::abs(2LL * vstart[cut] - nv)) cut = k;
+    bool shared = false;
+    const int t = border_tile(rel, vstart[cut], &shared);
+    if (t >= 0 && cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking) == cudaSuccess &&
+        cudaEventCreateWithFlags(&m->fork, cudaEventDisableTiming) == cudaSuccess &&
+        cudaEventCreateWithFlags(&m->join, cudaEventDisableTiming) == cudaSuccess) {
+      m->ngroup = 2;
+      m->group[0].v1 = m->group[1].v0 = vstart[cut];
+      m->group[1].v1 = nv;
+      m->group[0].tile1 = t + (shared ? 1 : 0);
+      m->group[1].tile0 = t;
+      m->group[1].tile1 = rel->tiles.ntiles;
+    }
+  }
+  cudaGetLastError();
   auto up = [](size_t n) { return (n + 127) / 128 * 128; };
-  const size_t b_cg = up(nseg * sizeof(MixedCg)), b_part = up(3 * (size_t)nseg * sizeof(double)),
-               b_res = up(nmesh * sizeof(MixedResult)), b_seg = up(nseg * sizeof(MixedSeg)),
-               b_first = up((grid + 1) * sizeof(int));
-  char* d = nullptr;
-  if (cudaMalloc(&m->slab, b_cg + b_part + b_res + b_seg + b_first + 128) != cudaSuccess) {
+  std::vector<MixedSeg> seg[2];
+  std::vector<int> first[2];
+  size_t total = up(nmesh * sizeof(MixedResult));
+  for (int g = 0; g < m->ngroup; ++g) {
+    cut_segments(vstart, m->group[g].v0, m->group[g].v1, grid, seg[g], first[g]);
+    const size_t n = seg[g].size();
+    m->group[g].nseg = (int)n;
+    total += up(n * sizeof(MixedCg)) + up(3 * n * sizeof(double)) + up(n * sizeof(MixedSeg)) +
+             up((grid + 1) * sizeof(int)) + 128;
+  }
+  if (cudaMalloc(&m->slab, total) != cudaSuccess) {
     m->slab = nullptr;
     cudaGetLastError();
     return false;
   }
-  d = static_cast<char*>(m->slab);
-  m->cg = reinterpret_cast<MixedCg*>(d);
-  m->part = reinterpret_cast<double*>(d += b_cg);
-  m->res = reinterpret_cast<MixedResult*>(d += b_part);
-  m->seg = reinterpret_cast<MixedSeg*>(d += b_res);
-  m->first = reinterpret_cast<int*>(d += b_seg);
-  m->ctl = reinterpret_cast<unsigned*>(d += b_first);
-  if (cudaMemcpy(m->seg, seg.data(), nseg * sizeof(MixedSeg), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(m->first, first.data(), (grid + 1) * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(m->slab);
-    m->slab = nullptr;
-    return false;
+  char* d = static_cast<char*>(m->slab);
+  auto take = [&](size_t n) {
+    char* at = d;
+    d += up(n);
+    return at;
+  };
+  m->res = reinterpret_cast<MixedResult*>(take(nmesh * sizeof(MixedResult)));
+  for (int g = 0; g < m->ngroup; ++g) {
+    MixedGroup& q = m->group[g];
+    const size_t n = q.nseg;
+    q.cg = reinterpret_cast<MixedCg*>(take(n * sizeof(MixedCg)));
+    q.part = reinterpret_cast<double*>(take(3 * n * sizeof(double)));
+    q.seg = reinterpret_cast<MixedSeg*>(take(n * sizeof(MixedSeg)));
+    q.first = reinterpret_cast<int*>(take((grid + 1) * sizeof(int)));
+    q.ctl = reinterpret_cast<unsigned*>(take(128));
+    if (cudaMemcpy(q.seg, seg[g].data(), n * sizeof(MixedSeg), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(q.first, first[g].data(), (grid + 1) * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(m->slab);
+      m->slab = nullptr;
+      return false;
+    }
   }
-  m->nmesh = nmesh;
-  m->nseg = nseg;
   m->grid = grid;
   return true;
 }
 
 cudaError_t launch_mixed_cg(ebb_rel_s* rel, MixedPlan* m, int model, float mu0, float lam0, const MixedVectors& v,
                             double dt, double rtol, int max_iters, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(m->ctl, 0, 2 * sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  MixedArgs a;
-  a.nv = (int)rel->verts->size;
-  a.ntiles = rel->tiles.ntiles;
-  a.blobs = rel->tiles.blob32;
-  a.L = rel->tiles.L32;
-  a.perm = rel->tet_perm;
-  a.mu0 = mu0;
-  a.lam0 = lam0;
-  a.err = rel->ctx->d_err;
-  a.v = v;
-  a.seg = m->seg;
-  a.first = m->first;
-  a.nseg = m->nseg;
-  a.cg = m->cg;
-  a.part = m->part;
-  a.res = m->res;
-  a.ctl = m->ctl;
-  a.dt = dt;
-  a.rtol = rtol;
-  a.max_iters = max_iters;
-  a.walker_smem = walker_bytes(a.L);
-  if (v.pin_bytes == 4)
-    return model == EBB_STVK ? launch<EBB_STVK, int>(a, m->grid, st) : launch<EBB_NEOHOOKEAN, int>(a, m->grid, st);
-  return model == EBB_STVK ? launch<EBB_STVK, unsigned char>(a, m->grid, st)
-                           : launch<EBB_NEOHOOKEAN, unsigned char>(a, m->grid, st);
+  cudaError_t e = cudaSuccess;
+  if (m->ngroup == 2) {
+    e = cudaEventRecord(m->fork, st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(m->side, m->fork, 0);
+  }
+  for (int g = 0; g < m->ngroup && e == cudaSuccess; ++g) {
+    const MixedGroup& q = m->group[g];
+    cudaStream_t gs = g == 0 ? st : m->side;
+    e = cudaMemsetAsync(q.ctl, 0, 2 * sizeof(unsigned), gs);
+    if (e != cudaSuccess) break;
+    MixedArgs a;
+    a.nv = (int)rel->verts->size;
+    a.ntiles = q.tile1 - q.tile0;
+    a.v_lo = q.v0;
+    a.v_span = (unsigned)(q.v1 - q.v0);
+    a.L = rel->tiles.L32;
+    a.blobs = rel->tiles.blob32 + (size_t)q.tile0 * a.L.bytes;
+    a.perm = rel->tet_perm;
+    a.mu0 = mu0;
+    a.lam0 = lam0;
+    a.err = rel->ctx->d_err;
+    a.v = v;
+    a.seg = q.seg;
+    a.first = q.first;
+    a.nseg = q.nseg;
+    a.cg = q.cg;
+    a.part = q.part;
+    a.res = m->res;
+    a.ctl = q.ctl;
+    a.dt = dt;
+    a.rtol = rtol;
+    a.max_iters = max_iters;
+    a.walker_smem = walker_bytes(a.L);
+    if (m->ngroup == 2)   // batches pin by bytes
+      e = model == EBB_STVK ? launch<Half, EBB_STVK, unsigned char>(a, m->grid, gs)
+                            : launch<Half, EBB_NEOHOOKEAN, unsigned char>(a, m->grid, gs);
+    else if (v.pin_bytes == 4)
+      e = model == EBB_STVK ? launch<One, EBB_STVK, int>(a, m->grid, gs)
+                            : launch<One, EBB_NEOHOOKEAN, int>(a, m->grid, gs);
+    else
+      e = model == EBB_STVK ? launch<One, EBB_STVK, unsigned char>(a, m->grid, gs)
+                            : launch<One, EBB_NEOHOOKEAN, unsigned char>(a, m->grid, gs);
+  }
+  if (m->ngroup == 2 && e == cudaSuccess) {
+    e = cudaEventRecord(m->join, m->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, m->join, 0);
+  }
+  return e;
 }
 
 }  // namespace ebb

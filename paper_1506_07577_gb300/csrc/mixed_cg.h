@@ -32,9 +32,10 @@ struct MixedPlan;
 bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vstart, MixedPlan** plan);
 void free_mixed_plan(MixedPlan* plan);
 
-// Solve on `st` (asynchronous) and the meshes' results on the device.
+// Solve, ordered after the work on `st` and before later work there (asynchronous).
+// The meshes' results are left on the device, one per mesh.
 cudaError_t launch_mixed_cg(ebb_rel_s* rel, MixedPlan* plan, int model, float mu0, float lam0, const MixedVectors& v,
                             double dt, double rtol, int max_iters, cudaStream_t st);
-const MixedResult* mixed_results(const MixedPlan* plan);   // device array, one per mesh
+const MixedResult* mixed_results(const MixedPlan* plan);
 
 }  // namespace ebb

@@ -491,9 +491,11 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
 #pragma unroll
           for (int f = 0; f < NF; ++f) st_part4(row + 4 * f, acc[f], acc[NF + f], acc[2 * NF + f]);
         } else if constexpr (AOS) {
+          if (OPS != OP_KV || (unsigned)(v - io.v_lo) < io.v_span) {
 #pragma unroll
-          for (int f = 0; f < NF; ++f)
-            red_add_v4(out_field[f] + 4 * (size_t)v, acc[f], acc[NF + f], acc[2 * NF + f]);
+            for (int f = 0; f < NF; ++f)
+              red_add_v4(out_field[f] + 4 * (size_t)v, acc[f], acc[NF + f], acc[2 * NF + f]);
+          }
         } else {
 #pragma unroll
           for (int c = 0; c < 3; ++c)
