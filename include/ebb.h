@@ -312,7 +312,9 @@ ebb_status_t ebb_map_tet_force_Kv(ebb_ctx_t ctx, ebb_rel_t tets, const char* u,
  * copies overlap the map (fully so when consecutive tiles touch nearly
  * consecutive rows, as after EBB_FINALIZE_RENUMBER_VERTS).  The chunk plan
  * is built on the first such call after finalize or a re-tiling (a copy of
- * the internal keys to the host).  The host buffers are borrowed for the call only; the
+ * the internal keys to the host).  Packed rows in page-locked buffers that the
+ * device reaches itself go in and out by kernels instead, chunk by chunk (1, 2 or 6
+ * chunks, by size), without copies or staging.  The host buffers are borrowed for the call only; the
  * device fields keep the copied and computed values afterwards.  Errors: as
  * ebb_map_tet_force_Kv (checked before anything is copied); EBB_ERR_ARG for
  * a null host buffer (with N_v > 0); EBB_ERR_PHASE if the device fields u

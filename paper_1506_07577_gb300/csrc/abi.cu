@@ -118,6 +118,7 @@ void free_host_plan(ebb_rel_s* r) {
 
 void free_tet_data(ebb_rel_s* r) {
   free_host_plan(r);
+  free_host_rows(r);
   cudaFree(r->xyz_stage);
   r->xyz_stage = nullptr;
   cudaFree(r->keys);
@@ -1029,6 +1030,19 @@ ebb_status_t ebb_map_tet_force_Kv_host(ebb_ctx_t ctx, ebb_rel_t tets, const char
   const bool xyz = (opts->flags & EBB_MAP_HOST_XYZ) != 0;
   if (xyz && (!x4 || f64))
     return set_error(ctx, EBB_ERR_ARG, "EBB_MAP_HOST_XYZ needs FP32 fields of EBB_F32X4 elements");
+  // The tiled map on fields it reads in place runs in chunks that overlap
+  // the copies; every other form copies everything in, maps, copies out.
+  const ebb_reduce_t reduce = resolve_tiled(tets, opts->reduce, opts->model, opts->precision);
+  const bool staged = !x4 && !f64 && tets->stage_interleaved;
+  // Packed rows the GPU reaches itself need neither copies nor staging.
+  if (xyz && bytes > 0 && reduce == EBB_REDUCE_TILED && !tets->vperm && !(opts->flags & EBB_MAP_TEST_DROP_TILE) &&
+      tets->tiles.ntiles > 0) {
+    if (cudaSetDevice(ctx->device) != cudaSuccess) return set_error(ctx, EBB_ERR_CUDA, "cudaSetDevice failed");
+    bool done = false;
+    s = host_map_rows(ctx, tets, dev, same_input, u_host, w_host, f_host, Kw_host, opts, &done);
+    if (s) return s;
+    if (done) return read_device_error(ctx);
+  }
   float* stage = nullptr;
   if (xyz && bytes > 0) {
     if (cudaSetDevice(ctx->device) != cudaSuccess) return set_error(ctx, EBB_ERR_CUDA, "cudaSetDevice failed");
@@ -1039,10 +1053,6 @@ ebb_status_t ebb_map_tet_force_Kv_host(ebb_ctx_t ctx, ebb_rel_t tets, const char
     }
     stage = tets->xyz_stage;
   }
-  // The tiled map on fields it reads in place runs in chunks that overlap
-  // the copies; every other form copies everything in, maps, copies out.
-  const ebb_reduce_t reduce = resolve_tiled(tets, opts->reduce, opts->model, opts->precision);
-  const bool staged = !x4 && !f64 && tets->stage_interleaved;
   if (bytes > 0 && reduce == EBB_REDUCE_TILED && !tets->vperm && !staged &&
       !(opts->flags & EBB_MAP_TEST_DROP_TILE) && tets->tiles.ntiles >= 2 * HostPlan::kChunks) {
     if (cudaSetDevice(ctx->device) != cudaSuccess) return set_error(ctx, EBB_ERR_CUDA, "cudaSetDevice failed");

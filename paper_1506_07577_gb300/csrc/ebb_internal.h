@@ -198,6 +198,7 @@ inline int chunk_first_tile(int c, int ntiles, int K) {
 struct BatchScratch;  // defined in batched.cu
 struct RowMatrix;     // defined in row_matrix.cuh
 struct RowStep;       // defined in row_step.cu
+struct HostRows;      // defined in host_rows.cu
 
 struct ebb_rel_impl;
 
@@ -247,6 +248,7 @@ struct ebb_rel_s {
   ebb::RowMatrix* rows = nullptr;       // row matrix pattern (row_matrix.cu), built on first use
   ebb::RowStep* row_step = nullptr;     // FP64 step on the rows (row_step.cu)
   ebb::HostPlan* hplan = nullptr;       // chunk plan of the host-buffer map (abi.cu)
+  ebb::HostRows* hrows = nullptr;       // and of its form on host rows the GPU reaches (host_rows.cu)
   float* xyz_stage = nullptr;           // host-buffer map's packed-row staging: u, w, f, Kw, 3 x N_v floats
                                         // each (EBB_MAP_HOST_XYZ; allocated on first use)
   ebb::BatchScratch* batch = nullptr;
@@ -427,6 +429,13 @@ cudaError_t launch_spmv(ebb_rel_s* rel, const T* w, T* y, bool aos, const int* a
 cudaError_t springs_init(ebb_rel_s* tets, const void* X, bool f64, cudaStream_t st);
 cudaError_t springs_run(ebb_rel_s* tets, void* q, void* qd, const void* mass, bool f64, double k, double dt, int steps,
                         double* energy, cudaStream_t st);
+
+// The host-buffer map on packed rows that the GPU reaches itself (host_rows.cu);
+// *done is false when it does not reach all four buffers.  Asynchronous on the
+// context's stream.
+ebb_status_t host_map_rows(ebb_ctx_s* ctx, ebb_rel_s* tets, void* const* dev, bool same_input, const void* u_host,
+                           const void* w_host, void* f_host, void* Kw_host, const ebb_map_opts_t* opts, bool* done);
+void free_host_rows(ebb_rel_s* tets);
 
 // Build the colouring (colour.cu).
 ebb_status_t build_colouring(ebb_ctx_s* ctx, ebb_rel_s* tets);
