@@ -189,6 +189,17 @@ bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb) {
   return pa < pb + nb && pb < pa + na;
 }
 
+// Host memory of plans built on first use (row pattern, solve segments, host-row
+// lists) runs out as an exception; it becomes a status here.
+template <typename F>
+ebb_status_t guarded(ebb_ctx_s* ctx, F call) {
+  try {
+    return call();
+  } catch (const std::bad_alloc&) {
+    return set_error(ctx, EBB_ERR_NOMEM, "host memory ran out");
+  }
+}
+
 // A concrete reduction variant (AUTO resolved).
 bool valid_reduce(int r) {
   return r == EBB_REDUCE_ATOMIC || r == EBB_REDUCE_COLOR || r == EBB_REDUCE_TILED || r == EBB_REDUCE_GATHER ||
@@ -1039,7 +1050,9 @@ ebb_status_t ebb_map_tet_force_Kv_host(ebb_ctx_t ctx, ebb_rel_t tets, const char
       tets->tiles.ntiles > 0) {
     if (cudaSetDevice(ctx->device) != cudaSuccess) return set_error(ctx, EBB_ERR_CUDA, "cudaSetDevice failed");
     bool done = false;
-    s = host_map_rows(ctx, tets, dev, same_input, u_host, w_host, f_host, Kw_host, opts, &done);
+    s = guarded(ctx, [&] {
+      return host_map_rows(ctx, tets, dev, same_input, u_host, w_host, f_host, Kw_host, opts, &done);
+    });
     if (s) return s;
     if (done) return read_device_error(ctx);
   }
@@ -1154,7 +1167,8 @@ ebb_status_t ebb_assemble_tet_K(ebb_ctx_t ctx, ebb_rel_t tets, const char* u, co
   mc.in[0] = u;
   mc.nin = 1;
   mc.nout = 0;
-  return run_map(ctx, tets, mc, OP_ASSEMBLE, opts);
+  if (!ctx) return EBB_ERR_ARG;
+  return guarded(ctx, [&] { return run_map(ctx, tets, mc, OP_ASSEMBLE, opts); });
 }
 
 ebb_status_t ebb_spmv_tet_K(ebb_ctx_t ctx, ebb_rel_t tets, const char* w, const char* Kw_out,
@@ -1411,7 +1425,7 @@ ebb_status_t ebb_cg_implicit_step(ebb_ctx_t ctx, ebb_rel_t tets, const char* u, 
   }
   ebb_step_params_t p = *params;
   p.reduce = reduce;
-  return run_implicit_step(ctx, tets, (double*)pu, (double*)pv, pp, pdt, &p, report);
+  return guarded(ctx, [&] { return run_implicit_step(ctx, tets, (double*)pu, (double*)pv, pp, pdt, &p, report); });
 }
 
 namespace {
@@ -1470,8 +1484,10 @@ ebb_status_t step_vjp_entry(ebb_ctx_t ctx, ebb_rel_t tets, const char* u, const 
   }
   ebb_step_params_t p = *params;
   p.reduce = reduce;
-  return run_step_vjp(ctx, tets, (const double*)pu, (const double*)pv, (const double*)pvn, pp, pdt, (double*)pgu,
-                      (double*)pgv, per_tet[0], per_tet[1], &p, report);
+  return guarded(ctx, [&] {
+    return run_step_vjp(ctx, tets, (const double*)pu, (const double*)pv, (const double*)pvn, pp, pdt, (double*)pgu,
+                        (double*)pgv, per_tet[0], per_tet[1], &p, report);
+  });
 }
 }  // namespace
 
@@ -1534,7 +1550,8 @@ ebb_status_t ebb_cg_implicit_step_batched(ebb_ctx_t ctx, ebb_rel_t tets, const c
   }
   ebb_step_params_t p = *params;
   p.reduce = reduce;
-  return run_batched_step(ctx, tets, (double*)pu, (double*)pv, pp, (const int*)pb, nbatch, &p, reports);
+  return guarded(
+      ctx, [&] { return run_batched_step(ctx, tets, (double*)pu, (double*)pv, pp, (const int*)pb, nbatch, &p, reports); });
 }
 
 }  // extern "C"
