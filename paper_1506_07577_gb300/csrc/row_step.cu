@@ -14,8 +14,10 @@
 // No atomics on floating-point data: results repeat bit for bit, whatever
 // reduction the caller names.
 // Measured, against the matrix-free step with two launches per iteration: 8^3
-// StVK step (2,560 tets) 498 -> 138 us; 20-step rollout and gradient on the
-// 32^3 mesh (163,840 tets) 213 -> 46 ms.
+// StVK step (2,560 tets) 504 -> 143 us; 20-step rollout and gradient on the
+// 32^3 mesh (163,840 tets) 212 -> 48 ms.  The small step's solve in one cluster
+// of 16 blocks, sums through distributed shared memory: 185 us, 16 SMs' FP64
+// pipes being too few.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -56,10 +58,11 @@ constexpr int kSplitThreads = 128;   // its form for few slices
 constexpr int kMaxGrid = kRowMaxGrid;   // partial sums per set
 
 // Streaming load of a matrix value (read once per product: not kept in L1,
-// which the gathered vector entries use).
+// which the gathered vector entries use). Not through the read-only path: the
+// kernel itself writes the diagonal blocks at its start.
 __device__ __forceinline__ double ld_stream(const double* p) {
   double x;
-  asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(x) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(x) : "l"(p));
   return x;
 }
 
