@@ -8,9 +8,8 @@
 // reproducible.  The diagonal block is minus the sum of its row's other
 // blocks (K annihilates translations), so 6 of the 16 corner pairs are
 // formed per tet, each once.  Measured on the 64^3 mesh (1.31 M tets, FP32):
-// records 77 us, rows 182 us, product 44 us; one atomic per block entry and
-// tet took 716 us.  Three slots per warp in the row pass: 223 us (fewer warps
-// to cover the records' latency).
+// records 80 us, rows 143 us, product 45 us; one atomic per block entry and
+// tet took 716 us.
 #include <algorithm>
 
 #include "row_matrix.cuh"
@@ -201,22 +200,74 @@ scan_kernel(int n, const int* __restrict__ in, int* out) {
   if (threadIdx.x == 0) out[n] = s_run;
 }
 
-// The rows' columns and contribution ranges in slot order; eight lanes per row.
+// The rows' columns in slot order; eight lanes per row.
 __global__ void __launch_bounds__(256)
 row_fill_kernel(int nv, const int* __restrict__ off, const int* __restrict__ len, const int* __restrict__ colv,
-                const int* __restrict__ colb, const int* __restrict__ place, const int* __restrict__ slice_off,
-                int* col, int2* crange, int* slot_slice) {
+                const int* __restrict__ place, const int* __restrict__ slice_off, int* col) {
   const int v = (blockIdx.x * 256 + threadIdx.x) >> 3, lane = threadIdx.x & 7;
   if (v >= nv) return;
-  const int c0 = 3 * off[v], c1 = 3 * off[v + 1], m = len[v] - 1;
+  const int c0 = 3 * off[v], m = len[v] - 1;
   const int sl = place[v] / kSliceRows, i = place[v] - sl * kSliceRows;
   const int q0 = slice_off[sl], nk = slice_off[sl + 1] - q0;
-  for (int k = lane; k < nk; k += 8) {
-    const size_t at = (size_t)(q0 + k) * kSliceRows + i;
-    const bool in = k > 0 && k <= m;
-    col[at] = in ? colv[c0 + k - 1] : v;
-    crange[at] = in ? make_int2(colb[c0 + k - 1], k < m ? colb[c0 + k] : c1) : make_int2(0, 0);
-    if (i == 0) slot_slice[q0 + k] = sl;   // by the slice's longest row
+  for (int k = lane; k < nk; k += 8)
+    col[(size_t)(q0 + k) * kSliceRows + i] = k > 0 && k <= m ? colv[c0 + k - 1] : v;
+}
+
+// Place of the first of n increasing columns that is >= v.
+__device__ __forceinline__ int lower_bound(const int* __restrict__ col, int n, int v) {
+  int lo = 0;
+  while (lo < n) {
+    const int mid = (lo + n) >> 1;
+    if (col[mid] < v)
+      lo = mid + 1;
+    else
+      n = mid;
+  }
+  return lo;
+}
+
+// Block pairs (RowMatrix::pairs) of the rows of each slice, one warp per slice:
+// first their number (FILL false), then the pairs.
+template <bool FILL>
+__global__ void __launch_bounds__(256)
+row_pair_kernel(int nslice, const int* __restrict__ row_of, const int* __restrict__ off, const int* __restrict__ len,
+                const int* __restrict__ colv, const int* __restrict__ colb, const int* __restrict__ place,
+                const int* __restrict__ slice_off, int* count, const int* __restrict__ pair_off, int4* pairs) {
+  const int s = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (s >= nslice) return;
+  const int v = lane < kSliceRows ? row_of[s * kSliceRows + lane] : -1;
+  int c0 = 0, m = 0, lo = 0;
+  if (v >= 0) {
+    c0 = 3 * off[v];
+    m = len[v] - 1;
+    lo = lower_bound(colv + c0, m, v);
+  }
+  const int n = m - lo;
+  int inc = n;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if constexpr (!FILL) {
+    if (lane == 31) count[s] = inc;
+  } else {
+    const int base = pair_off[s] + inc - n;
+    for (int i = 0; i < kSliceRows; ++i) {
+      const int vi = __shfl_sync(0xffffffffu, v, i), ci = __shfl_sync(0xffffffffu, c0, i);
+      const int mi = __shfl_sync(0xffffffffu, m, i), li = __shfl_sync(0xffffffffu, lo, i);
+      const int bi = __shfl_sync(0xffffffffu, base, i);
+      for (int k = li + lane; k < mi; k += 32) {
+        const int w = colv[ci + k];
+        int mate = -1;
+        if (w != vi) {
+          const int pw = place[w], sw = pw / kSliceRows;
+          const int kw = lower_bound(colv + 3 * off[w], len[w] - 1, vi);
+          mate = (slice_off[sw] + 1 + kw) * kSliceRows + pw - sw * kSliceRows;
+        }
+        pairs[bi + k - li] = make_int4((slice_off[s] + 1 + k) * kSliceRows + i, mate, colb[ci + k],
+                                       k + 1 < mi ? colb[ci + k + 1] : 3 * off[vi + 1]);
+      }
+    }
   }
 }
 
@@ -449,33 +500,55 @@ namespace {
 
 constexpr int kAsmThreads = 256;
 
-// Off-diagonal blocks of scale * K, one warp per slot, a lane per row and
-// component: the sum of the block's contributions in increasing tet order.
-// Blocks of a record are stored for a < b; the other way round they are
-// transposed.  FP32: a lane loads its row of the stored block, one 16-byte load
-// per contribution (the loads' lines bound the kernel: with one load per entry
-// or nine lanes per block it took 3 times as long), adds stored and transposed
-// contributions apart and swaps the transposed sums between its row's lanes at the
-// end.  FP64: the adds bound it, so transposed entries are loaded as such.
+// Column c of a 3x3 block whose row c this lane holds, rows in lanes row0 + c.
+template <typename T>
+__device__ __forceinline__ void transpose3(const T (&x)[3], int c, int row0, T (&y)[3]) {
+  // lane c gets entry c of lanes c + 1 and c + 2 (mod 3)
+  const int n1 = c == 2 ? 0 : c + 1, n2 = c == 0 ? 2 : c - 1;
+  const T give1 = c == 0 ? x[2] : (c == 1 ? x[0] : x[1]);
+  const T give2 = c == 0 ? x[1] : (c == 1 ? x[2] : x[0]);
+  const T own = c == 0 ? x[0] : (c == 1 ? x[1] : x[2]);
+  const T got1 = __shfl_sync(0xffffffffu, give1, row0 + n1);
+  const T got2 = __shfl_sync(0xffffffffu, give2, row0 + n2);
+  y[0] = c == 0 ? own : (c == 1 ? got2 : got1);
+  y[1] = c == 1 ? own : (c == 2 ? got2 : got1);
+  y[2] = c == 2 ? own : (c == 0 ? got2 : got1);
+}
+
+// Off-diagonal blocks of scale * K, ten block pairs per warp, a lane per row of
+// the first block: the sum of the pair's contributions in increasing tet order,
+// stored as it is and, transposed, at its mate's place.  K is symmetric, and both
+// orders would add the same values in the same order.  Blocks of a record are
+// stored for a < b; the other way round they are transposed.  FP32: a lane loads
+// its row of the stored block, one 16-byte load per contribution (the loads'
+// lines bound the kernel: with one load per entry or nine lanes per block it took
+// 3 times as long), adds stored and transposed contributions apart and swaps the
+// transposed sums between its row's lanes at the end.  FP64: the adds bound it,
+// so transposed entries are loaded as such.  Measured against each block summed
+// by itself: 64^3 mesh, FP32 182 -> 143 us (160 with the mates stored entry by
+// entry, 30 sectors a store instead of 10); 32^3 mesh, FP64 73 -> 38 us.
 template <typename T, typename PT>
 __global__ void __launch_bounds__(kAsmThreads)
-row_block_kernel(int64_t nslots, const int* __restrict__ slice_off, const int* __restrict__ slot_slice,
-                 const int* __restrict__ row_of, const int2* __restrict__ crange, const int* __restrict__ contrib,
-                 const T* __restrict__ elem, const PT* __restrict__ pin, T scale, T* __restrict__ val) {
-  const int64_t q = ((int64_t)blockIdx.x * kAsmThreads + threadIdx.x) >> 5;
+row_block_kernel(int npair, const int4* __restrict__ pairs, const int* __restrict__ col,
+                 const int* __restrict__ contrib, const T* __restrict__ elem, const PT* __restrict__ pin, T scale,
+                 T* __restrict__ val) {
+  const int64_t warp = ((int64_t)blockIdx.x * kAsmThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (q >= nslots) return;
-  const int s = slot_slice[q];
-  const bool own = lane < 3 * kSliceRows;
-  const int i = own ? lane / 3 : 0, c = own ? lane - 3 * i : 0;
-  int2 r = own ? crange[q * kSliceRows + i] : make_int2(0, 0);
-  if (q == slice_off[s]) return;   // the diagonal blocks are not stored here
-  if (pin != nullptr && r.x < r.y && pin[row_of[s * kSliceRows + i]] != 0) r.y = r.x;
+  const int i = lane / 3, c = lane - 3 * i;
+  const int64_t n = warp * kSliceRows + i;
+  const bool own = lane < 3 * kSliceRows && n < npair;
+  int4 p = own ? pairs[n] : make_int4(0, -1, 0, 0);
+  bool zero = false, zero_mate = false;   // rows of pinned vertices
+  if (pin != nullptr && own) {
+    zero_mate = pin[col[p.x]] != 0;
+    zero = p.y >= 0 ? pin[col[p.y]] != 0 : zero_mate;
+    if (zero && zero_mate) p.w = p.z;
+  }
   T x[3] = {T(0), T(0), T(0)};
   if constexpr (sizeof(T) == 4) {
     T xt[3] = {T(0), T(0), T(0)};
 #pragma unroll 4
-    for (int e = r.x; e < r.y; ++e) {
+    for (int e = p.z; e < p.w; ++e) {
       const int code = contrib[e];
       const float4 k = __ldg(reinterpret_cast<const float4*>(elem + (size_t)(code >> 4) * kElemLen +
                                                              12 * ((code >> 1) & 7) + 4 * c));
@@ -489,34 +562,41 @@ row_block_kernel(int64_t nslots, const int* __restrict__ slice_off, const int* _
         x[2] += k.z;
       }
     }
-    // lane c's entry d of the transposed sum is lane d's entry c
-    const int row0 = lane - c;
+    T y[3];
+    transpose3(xt, c, lane - c, y);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      T y[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) y[k] = __shfl_sync(0xffffffffu, xt[k], row0 + d);
-      x[d] += c == 0 ? y[0] : (c == 1 ? y[1] : y[2]);
-    }
-  } else if (r.x < r.y) {
+    for (int d = 0; d < 3; ++d) x[d] += y[d];
+  } else if (p.z < p.w) {
     auto rec_of = [&](int code, int& st) {
       const bool tr = (code & 1) != 0;
       st = tr ? 4 : 1;
       return elem + (size_t)(code >> 4) * kElemLen + 12 * ((code >> 1) & 7) + (tr ? c : 4 * c);
     };
     int st;
-    const T* rec = rec_of(contrib[r.x], st);
+    const T* rec = rec_of(contrib[p.z], st);
 #pragma unroll
     for (int d = 0; d < 3; ++d) x[d] = rec[d * st];
 #pragma unroll 4
-    for (int e = r.x + 1; e < r.y; ++e) {
+    for (int e = p.z + 1; e < p.w; ++e) {
       rec = rec_of(contrib[e], st);
 #pragma unroll
       for (int d = 0; d < 3; ++d) x[d] += rec[d * st];
     }
   }
+  T y[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) val[((size_t)q * 3 + d) * 32 + lane] = scale * x[d];
+  for (int d = 0; d < 3; ++d) x[d] *= scale;
+  transpose3(x, c, lane - c, y);
+  if (!own) return;
+  const int q = p.x / kSliceRows;
+  T* at = val + (size_t)q * 96 + 3 * (p.x - q * kSliceRows) + c;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) at[32 * d] = zero ? T(0) : x[d];
+  if (p.y < 0) return;
+  const int qm = p.y / kSliceRows;
+  at = val + (size_t)qm * 96 + 3 * (p.y - qm * kSliceRows) + c;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) at[32 * d] = zero_mate ? T(0) : y[d];
 }
 
 __device__ __forceinline__ float ld_once(const float* p) {
@@ -591,16 +671,15 @@ row_product_kernel(RowView m, int nv, const T* __restrict__ val, const T* __rest
 template <typename T>
 cudaError_t launch_row_blocks(const RowMatrix& m, const T* elem, const void* pin, int pin_bytes, T scale, T* val,
                               cudaStream_t st) {
-  const int64_t grid = (m.nslots * 32 + kAsmThreads - 1) / kAsmThreads;
-  if (grid == 0) return cudaSuccess;
+  if (m.npair == 0) return cudaSuccess;
+  const int64_t warps = ((int64_t)m.npair + kSliceRows - 1) / kSliceRows;
+  const unsigned grid = (unsigned)((warps * 32 + kAsmThreads - 1) / kAsmThreads);
   if (pin_bytes == 4)
-    row_block_kernel<T, int><<<(unsigned)grid, kAsmThreads, 0, st>>>(m.nslots, m.slice_off, m.slot_slice, m.row_of,
-                                                                     m.crange, m.contrib, elem,
-                                                                     static_cast<const int*>(pin), scale, val);
+    row_block_kernel<T, int><<<grid, kAsmThreads, 0, st>>>(m.npair, m.pairs, m.col, m.contrib, elem,
+                                                           static_cast<const int*>(pin), scale, val);
   else
-    row_block_kernel<T, unsigned char><<<(unsigned)grid, kAsmThreads, 0, st>>>(
-        m.nslots, m.slice_off, m.slot_slice, m.row_of, m.crange, m.contrib, elem,
-        static_cast<const unsigned char*>(pin), scale, val);
+    row_block_kernel<T, unsigned char><<<grid, kAsmThreads, 0, st>>>(
+        m.npair, m.pairs, m.col, m.contrib, elem, static_cast<const unsigned char*>(pin), scale, val);
   return cudaGetLastError();
 }
 template cudaError_t launch_row_blocks<double>(const RowMatrix&, const double*, const void*, int, double, double*,
@@ -624,8 +703,10 @@ cudaError_t launch_row_assemble(ebb_rel_s* rel, int model, T mu0, T lam0, const 
     if (m->state != 1) return cudaSuccess;
     e = cudaMalloc(&m->val[p], std::max<size_t>(1, (size_t)m->nslots * 96) * sizeof(T));
     if (e == cudaSuccess) e = cudaMalloc(&m->elem[p], std::max<size_t>(1, (size_t)rel->size * kElemLen) * sizeof(T));
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->val[p], 0, (size_t)m->nslots * 96 * sizeof(T), st);   // unused entries
     if (e != cudaSuccess) {
       cudaFree(m->val[p]);
+      cudaFree(m->elem[p]);
       m->val[p] = m->elem[p] = nullptr;
       cudaGetLastError();
       return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
@@ -686,8 +767,7 @@ void free_row_matrix(ebb_rel_s* tets) {
   cudaFree(m->slice_off);
   cudaFree(m->row_of);
   cudaFree(m->col);
-  cudaFree(m->crange);
-  cudaFree(m->slot_slice);
+  cudaFree(m->pairs);
   cudaFree(m->contrib);
   for (int p = 0; p < 2; ++p) {
     cudaFree(m->val[p]);
@@ -710,7 +790,7 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
   m->nslice = nwin * kWindowSlices;
   // scratch: row lengths, places, slot counts, the too-long flag, columns
   int* tmp = nullptr;
-  const size_t ntmp = 2 * (size_t)nv + m->nslice + 1 + (size_t)nt * 24;
+  const size_t ntmp = 2 * (size_t)nv + 2 * (size_t)m->nslice + 2 + (size_t)nt * 24;
   cudaError_t e = cudaMalloc(&tmp, ntmp * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&m->slice_off, ((size_t)m->nslice + 1) * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&m->row_of, (size_t)nwin * kWindowRows * sizeof(int));
@@ -720,7 +800,7 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
   m->grid = std::min({std::max(nsm, 1), kRowMaxGrid, m->nslice});
   int host[2] = {0, 0};   // total slots, too-long flag
   int *len = tmp, *place = tmp + nv, *slots = tmp + 2 * (size_t)nv, *flag = slots + m->nslice;
-  int *colv = flag + 1, *colb = colv + (size_t)nt * 12;
+  int *pair_off = flag + 1, *colv = pair_off + m->nslice + 1, *colb = colv + (size_t)nt * 12;
   if (e == cudaSuccess) {
     const VertexIndex& x = tets->vindex;
     e = cudaMemsetAsync(flag, 0, sizeof(int), st);
@@ -737,19 +817,29 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
     if (e == cudaSuccess) e = cudaMemcpyAsync(&host[1], flag, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
-  bool apply = e == cudaSuccess && host[1] == 0;
+  // places of entries are 32-bit
+  bool apply = e == cudaSuccess && host[1] == 0 && host[0] <= 0x7fffffff / kSliceRows;
   if (apply) {
     m->nslots = host[0];
     const size_t n = std::max<size_t>(1, (size_t)m->nslots * kSliceRows);
+    const int sg = (m->nslice * 32 + 255) / 256;
     e = cudaMalloc(&m->col, n * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&m->crange, n * sizeof(int2));
-    if (e == cudaSuccess) e = cudaMalloc(&m->slot_slice, std::max<size_t>(1, (size_t)m->nslots) * sizeof(int));
-    // rows that hold no vertex: a valid column, no contributions
+    // rows that hold no vertex: a valid column
     if (e == cudaSuccess) e = cudaMemsetAsync(m->col, 0, n * sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->crange, 0, n * sizeof(int2), st);
     if (e == cudaSuccess) {
-      row_fill_kernel<<<(nv + 31) / 32, 256, 0, st>>>(nv, tets->vindex.off, len, colv, colb, place, m->slice_off,
-                                                      m->col, m->crange, m->slot_slice);
+      row_fill_kernel<<<(nv + 31) / 32, 256, 0, st>>>(nv, tets->vindex.off, len, colv, place, m->slice_off, m->col);
+      row_pair_kernel<false><<<sg, 256, 0, st>>>(m->nslice, m->row_of, tets->vindex.off, len, colv, colb, place,
+                                                 m->slice_off, slots, nullptr, nullptr);
+      scan_kernel<<<1, kScanThreads, 0, st>>>(m->nslice, slots, pair_off);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&m->npair, pair_off + m->nslice, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = cudaMalloc(&m->pairs, std::max<size_t>(1, (size_t)m->npair) * sizeof(int4));
+    if (e == cudaSuccess) {
+      row_pair_kernel<true><<<sg, 256, 0, st>>>(m->nslice, m->row_of, tets->vindex.off, len, colv, colb, place,
+                                                m->slice_off, slots, pair_off, m->pairs);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -760,10 +850,9 @@ ebb_status_t ensure_row_pattern(ebb_ctx_s* ctx, ebb_rel_s* tets, cudaStream_t st
     cudaFree(m->slice_off);
     cudaFree(m->row_of);
     cudaFree(m->col);
-    cudaFree(m->crange);
-    cudaFree(m->slot_slice);
+    cudaFree(m->pairs);
     cudaFree(m->contrib);
-      *m = RowMatrix();
+    *m = RowMatrix();
     m->state = -1;
     if (e == cudaSuccess || e == cudaErrorMemoryAllocation) {
       cudaGetLastError();

@@ -46,8 +46,10 @@ struct RowMatrix {
   int* slice_off = nullptr;   // nslice + 1
   int* row_of = nullptr;      // nslice * kSliceRows: vertex of each row, -1 for none
   int* col = nullptr;         // nslots * kSliceRows
-  int2* crange = nullptr;     // nslots * kSliceRows: the block's contributions [x, y)
-  int* slot_slice = nullptr;  // nslots: slice of each slot
+  // Blocks (v, w), w >= v, slice by slice: x the place of (v, w) as in col, y that
+  // of (w, v) (-1 when w is v), [z, w) its contributions.
+  int npair = 0;
+  int4* pairs = nullptr;
   int* contrib = nullptr;     // 12 per tet, row by row: 16 t + 2 pair + transposed
   bool no_step = false;       // the FP64 step's buffers did not fit (row_step.cu)
   int grid = 0;               // thread blocks of a kernel over all slices (at most one per SM)
@@ -84,7 +86,8 @@ cudaError_t launch_element_blocks(ebb_rel_s* rel, int model, T mu0, T lam0, cons
                                   cudaStream_t st);
 
 // Off-diagonal blocks of scale * K, zero on the rows of pinned vertices (pin may
-// be null; pin_bytes 1 or 4), from the element records.
+// be null; pin_bytes 1 or 4), from the element records.  Unused entries of val are
+// left as they are: its owner zeroes them once.
 template <typename T>
 cudaError_t launch_row_blocks(const RowMatrix& m, const T* elem, const void* pin, int pin_bytes, T scale, T* val,
                               cudaStream_t st);

@@ -14,8 +14,8 @@
 // No atomics on floating-point data: results repeat bit for bit, whatever
 // reduction the caller names.
 // Measured, against the matrix-free step with two launches per iteration: 8^3
-// StVK step (2,560 tets) 504 -> 143 us; 20-step rollout and gradient on the
-// 32^3 mesh (163,840 tets) 212 -> 48 ms.  The small step's solve in one cluster
+// StVK step (2,560 tets) 504 -> 137 us; 20-step rollout and gradient on the
+// 32^3 mesh (163,840 tets) 213 -> 46.7 ms.  The small step's solve in one cluster
 // of 16 blocks, sums through distributed shared memory: 185 us, 16 SMs' FP64
 // pipes being too few.
 #include <algorithm>
@@ -547,6 +547,13 @@ ebb_status_t ensure_row_step(ebb_ctx_s* ctx, ebb_rel_s* tets, bool* fits) {
   s->mass = take(nv);
   s->part = take(2 * kSums * kMaxGrid);
   s->bar = reinterpret_cast<unsigned*>(take(2));
+  e = cudaMemsetAsync(s->val, 0, val * sizeof(double), ctx->stream);   // unused entries stay zero
+  if (e != cudaSuccess) {
+    cudaFree(s->slab);
+    cudaFreeHost(s->host);
+    delete s;
+    return cuda_check(ctx, e, "implicit-step scratch");
+  }
   tets->row_step = s;
   return EBB_OK;
 }
