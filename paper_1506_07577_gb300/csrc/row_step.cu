@@ -203,8 +203,10 @@ __device__ __forceinline__ bool grid_sum(RowCgShared<NP>& sh, const double (&x)[
 // so all vectors but z stay with their thread: in registers for the warp's
 // first slice (all of them on meshes of up to 36,000 vertices), in memory for
 // the others.  SPLIT: four warps share a slice's slots and the first adds
-// their sums; for meshes with at most three slices per SM, where one warp's
-// chain of FP64 operations (64 cycles each) would be the iteration.
+// their sums; for meshes with at most two slices per SM, where one warp's chain
+// of FP64 operations (64 cycles each) would be the iteration.  Whole steps, split
+// and not: 12^3 mesh (1.4 slices per SM) 142 and 164 us, 13^3 (1.8) 142 and 162,
+// 14^3 (2.2) 186 and 175, 16^3 (3.2) 230 and 184.
 template <int NT, bool SPLIT, typename PT>
 __global__ void __launch_bounds__(NT, 1) row_cg_kernel(RowCgArgs a, const PT* __restrict__ pin) {
   constexpr int NP = SPLIT ? 32 : NT;
@@ -502,7 +504,7 @@ cudaError_t launch_cg(const RowCgArgs& a, const PT* pin, int grid, cudaStream_t 
 template <typename PT>
 cudaError_t solve(const RowCgArgs& a, const PT* pin, int grid, cudaStream_t st) {
   const int slices = (a.nv + kSliceRows - 1) / kSliceRows;   // that hold rows
-  if (slices <= 3 * grid) return launch_cg<kSplitThreads, true, PT>(a, pin, grid, st);
+  if (slices <= 2 * grid) return launch_cg<kSplitThreads, true, PT>(a, pin, grid, st);
   return launch_cg<kPlainThreads, false, PT>(a, pin, grid, st);
 }
 
