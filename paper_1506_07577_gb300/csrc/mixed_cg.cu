@@ -583,9 +583,12 @@ bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vsta
   // A block per SM and group: small meshes too, for whose few vertices and tiles
   // more SMs mean shorter passes.
   const int grid = nsm;
-  // Segments are summed one after the other: a batch of very many meshes is better
-  // off with a block per mesh.
-  if (nmesh > 16 * grid) return false;
+  // Segments are summed one after the other: a batch of very many small meshes is
+  // better off with a block per mesh.  Whole steps, one launch and separate ones, of
+  // 300, 450, 600 and 1000 meshes of 27 vertices: 222 and 248, 261 and 259, 290 and
+  // 278, 462 and 394 us; of 600 and 1000 meshes of 125 vertices: 327 and 344, 520 and
+  // 488 us; of 729 vertices: 772 and 879, 1299 and 1372 us.
+  if (nmesh > 16 * grid || (nmesh > 3 * grid && nv / nmesh < 512)) return false;
   const size_t walker = walker_bytes(rel->tiles.L32);
   if (!resident<One, EBB_STVK, unsigned char>(walker, 1) || !resident<One, EBB_NEOHOOKEAN, unsigned char>(walker, 1) ||
       !resident<One, EBB_STVK, int>(walker, 1) || !resident<One, EBB_NEOHOOKEAN, int>(walker, 1)) {
