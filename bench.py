@@ -63,8 +63,8 @@ G = (0.0, 0.0, -9.81)
 # record layout (`--profile --n 128 --permute --renumber --model stvk
 # --uniform --x4 [--planes]`).  They describe the kernel sources whose hash
 # is given and are reported as null (with a note) once those sources change.
-NCU_TRAFFIC = {"sources_sha256_16": "a1326421e942d5ff", "n": 128,
-               "bytes_per_launch": {"rows": 989.13e6, "planes": 904.88e6}}
+NCU_TRAFFIC = {"sources_sha256_16": "64f72dee4f227560", "n": 128,
+               "bytes_per_launch": {"rows": 989.70e6, "planes": 904.51e6}}
 # FP64 arithmetic of the FP64 kernels, counted by ncu (2 x DFMA + DADD + DMUL
 # thread instructions per unit) on the 64^3 workload, valid while the map and
 # spring sources hash to the same value.
