@@ -436,7 +436,8 @@ ebb_status_t ebb_ctx_create(ebb_ctx_t* out, int device, void* cuda_stream) {
   ctx->stream = (cudaStream_t)cuda_stream;
   if (cudaSetDevice(device) != cudaSuccess || cudaMalloc(&ctx->d_err, ERRW_WORDS * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&ctx->h_err, ERRW_WORDS * sizeof(int)) != cudaSuccess ||
-      cudaMemset(ctx->d_err, 0, ERRW_WORDS * sizeof(int)) != cudaSuccess) {
+      cudaMemsetAsync(ctx->d_err, 0, ERRW_WORDS * sizeof(int), cudaStreamLegacy) != cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
     cudaFree(ctx->d_err);
     if (ctx->h_err) cudaFreeHost(ctx->h_err);
     delete ctx;
@@ -646,10 +647,13 @@ static ebb_status_t relation_finalize(ebb_rel_t tets, uint32_t flags) {
       tets->vorder = vp;
     } else {
       ve = cudaMalloc(&tets->vperm, sizeof(int) * nv);
-      if (ve == cudaSuccess) ve = cudaMemcpy(tets->vperm, vp.data(), sizeof(int) * nv, cudaMemcpyHostToDevice);
+      if (ve == cudaSuccess)
+        ve = cudaMemcpyAsync(tets->vperm, vp.data(), sizeof(int) * nv, cudaMemcpyHostToDevice, ctx->stream);
     }
     if (ve == cudaSuccess) ve = cudaMalloc(&X_int, sizeof(double) * hX.size());
-    if (ve == cudaSuccess) ve = cudaMemcpy(X_int, hX.data(), sizeof(double) * hX.size(), cudaMemcpyHostToDevice);
+    if (ve == cudaSuccess)
+      ve = cudaMemcpyAsync(X_int, hX.data(), sizeof(double) * hX.size(), cudaMemcpyHostToDevice, ctx->stream);
+    if (ve == cudaSuccess) ve = cudaStreamSynchronize(ctx->stream);
     if (ve != cudaSuccess) {
       cudaFree(X_int);
       free_tet_data(tets);

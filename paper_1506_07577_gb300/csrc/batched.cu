@@ -440,7 +440,10 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   host.insert(host.end(), blk_v1.begin(), blk_v1.end());
   host.insert(host.end(), mesh_blk0.begin(), mesh_blk0.end());
   host.insert(host.end(), mesh_nblk.begin(), mesh_nblk.end());
-  e = cudaMemcpy(s->table, host.data(), sizeof(int) * host.size(), cudaMemcpyHostToDevice);
+  // on the solve's stream: a copy from pageable memory may return before it has
+  // landed, and this stream does not wait for the legacy default one
+  e = cudaMemcpyAsync(s->table, host.data(), sizeof(int) * host.size(), cudaMemcpyHostToDevice, s->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) {
     free_batch_scratch(tets);
     return cuda_check(ctx, e, "uploading the batch table");

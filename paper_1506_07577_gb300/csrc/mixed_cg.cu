@@ -649,8 +649,15 @@ bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vsta
     q.seg = reinterpret_cast<MixedSeg*>(take(n * sizeof(MixedSeg)));
     q.first = reinterpret_cast<int*>(take((grid + 1) * sizeof(int)));
     q.ctl = reinterpret_cast<unsigned*>(take(128));
-    if (cudaMemcpy(q.seg, seg[g].data(), n * sizeof(MixedSeg), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(q.first, first[g].data(), (grid + 1) * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) {
+    // On the context's stream, which the solve's streams follow: a copy from pageable
+    // memory may return before it has landed, and none of them waits for the legacy
+    // default stream.
+    cudaStream_t up_st = ctx->stream;
+    cudaError_t e = cudaMemcpyAsync(q.seg, seg[g].data(), n * sizeof(MixedSeg), cudaMemcpyHostToDevice, up_st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(q.first, first[g].data(), (grid + 1) * sizeof(int), cudaMemcpyHostToDevice, up_st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(up_st);
+    if (e != cudaSuccess) {
       cudaGetLastError();
       cudaFree(m->slab);
       m->slab = nullptr;
