@@ -132,7 +132,10 @@ spring_load_kernel(int nv, int nrows, const int* __restrict__ row_of, const T* _
 // position loads; FP64: by the FP64 pipe.  The last step writes positions and
 // velocities to the caller's planes.  Steps are launched to overlap: a step's
 // blocks take the places of the last step's as these end, read what no step
-// writes, and wait for the last step's positions then.  Measured per FP32 step on
+// writes, and wait for the last step's positions then.  Positions and velocities
+// are therefore plain pointers: another launch may still be writing them when this
+// one starts, so they are not constant during the kernel, as __restrict__ on a
+// read-only pointer would promise (and allow loads that skip coherence).  Measured per FP32 step on
 // the 64^3 mesh (274,625 vertices, 3.2 M directed springs): 9.3 us; groups of 4
 // or 9 springs, or more blocks with fewer registers, 10 to 15 us; a thread walking
 // its row of the edge relation, 17.1 us.
@@ -141,8 +144,8 @@ constexpr int kStepThreads = 128, kStepGroup = 6;
 template <typename T>
 __global__ void __launch_bounds__(kStepThreads, sizeof(T) == 4 ? 8 : 4)
 spring_step_kernel(int nv, int nslice, const int* __restrict__ row_of, const int* __restrict__ slice_off,
-                   const int* __restrict__ end, const T* __restrict__ rest, T k, T dt, const Quad<T>* __restrict__ qin,
-                   Quad<T>* __restrict__ qout, Quad<T>* __restrict__ vel, T* q_planes, T* qd_planes) {
+                   const int* __restrict__ end, const T* __restrict__ rest, T k, T dt, const Quad<T>* qin,
+                   Quad<T>* qout, Quad<T>* vel, T* q_planes, T* qd_planes) {
   release_next_kernel();
   const int r = blockIdx.x * kStepThreads + threadIdx.x;
   const int s = r >> 5, lane = r & 31;
