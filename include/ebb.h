@@ -529,8 +529,11 @@ ebb_status_t ebb_cg_implicit_step_vjp_at(ebb_ctx_t ctx, ebb_rel_t tets, const ch
  * id in [0, nbatch); ids must be non-decreasing along verts (each mesh's
  * vertices contiguous) and every id must occur.  Bind the field as
  * "batch" before ebb_relation_finalize so tets are ordered mesh by mesh and
- * a tet joining two meshes is rejected (EBB_ERR_KEY).  Every element map
- * runs as one launch over all meshes; CG scalars, convergence and iteration
+ * a tet joining two meshes is rejected (EBB_ERR_KEY); with ids bound later,
+ * or others than those, the results are the same and the tets' order costs
+ * locality and the split below.  Every element map
+ * runs over all meshes at once (mixed-precision solves of tets ordered mesh by
+ * mesh as two groups of meshes side by side); CG scalars, convergence and iteration
  * counts are per mesh (a converged mesh stops updating while others go on).
  * `pinned` must be a U8 field or NULL.  reports (may be NULL) receives nbatch
  * entries.  Synchronous.  Returns the first failing mesh's status (its

@@ -463,54 +463,54 @@ bool resident(size_t walker, int want) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, SH::threads, smem) == cudaSuccess && n >= want;
 }
 
-// First tile that holds a tet of vertices >= v (the tets of a batch are ordered
-// mesh by mesh) and whether it also holds a tet before, by one thread: out[0], out[1].
-__global__ void border_kernel(const int4* __restrict__ keys, int nt, const unsigned char* __restrict__ blobs,
-                              int blob_bytes, int ntiles, int v, int* out) {
-  int lo = 0, hi = nt;
-  while (lo < hi) {
-    const int m = lo + (hi - lo) / 2;
-    if (keys[m].x < v)
-      lo = m + 1;
-    else
-      hi = m;
+// Where the tiles of the vertices < v and those of the vertices >= v part: the last
+// tile with a tet of the former, the first with a tet of the latter, and whether a tet
+// joins both.  Every tet is looked at: the tets lie mesh by mesh only when the same ids
+// were the "batch" field of finalize, and a step takes any field.
+struct Border {
+  int last, first, joined;
+};
+
+__global__ void __launch_bounds__(kTileTets)
+border_kernel(const int4* __restrict__ keys, const unsigned char* __restrict__ blobs, int blob_bytes, int ntiles, int v,
+              Border* out) {
+  int last = -1, first = ntiles;
+  bool joined = false;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int4 h = *reinterpret_cast<const int4*>(blobs + (size_t)tile * blob_bytes);   // tets, slots, first tet
+    if ((int)threadIdx.x >= h.x) continue;
+    const int4 k = keys[h.z + threadIdx.x];
+    const bool below = min(min(k.x, k.y), min(k.z, k.w)) < v, above = max(max(k.x, k.y), max(k.z, k.w)) >= v;
+    if (below) last = tile;
+    if (above) first = min(first, tile);
+    joined |= below && above;
   }
-  const int tet = lo;
-  out[0] = ntiles;
-  out[1] = 0;
-  if (tet >= nt) return;
-  auto first_tet = [&](int tile) { return reinterpret_cast<const int4*>(blobs + (size_t)tile * blob_bytes)->z; };
-  lo = 0;
-  hi = ntiles;   // the last tile whose first tet is <= tet
-  while (hi - lo > 1) {
-    const int m = (lo + hi) / 2;
-    if (first_tet(m) <= tet)
-      lo = m;
-    else
-      hi = m;
-  }
-  out[0] = lo;
-  out[1] = first_tet(lo) < tet ? 1 : 0;
+  last = __reduce_max_sync(0xffffffffu, last);
+  first = __reduce_min_sync(0xffffffffu, first);
+  joined = __any_sync(0xffffffffu, joined);
+  if ((threadIdx.x & 31) != 0) return;
+  if (last >= 0) atomicMax(&out->last, last);
+  if (first < ntiles) atomicMin(&out->first, first);
+  if (joined) out->joined = 1;
 }
 
-// That on the host; -1 when a call fails.
-int border_tile(ebb_rel_s* rel, int v, bool* mixed, cudaStream_t st) {
-  int* d = nullptr;
-  int h[2] = {-1, 0};
-  cudaError_t e = cudaMalloc(&d, 2 * sizeof(int));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return -1;
+// That on the host; false when a call fails.
+bool find_border(ebb_rel_s* rel, int v, Border* b, cudaStream_t st) {
+  const int ntiles = rel->tiles.ntiles;
+  *b = Border{-1, ntiles, 0};
+  Border* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, sizeof(Border));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d, b, sizeof(Border), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    border_kernel<<<std::min(ntiles, 2432), kTileTets, 0, st>>>(rel->keys, rel->tiles.blob32, rel->tiles.L32.bytes,
+                                                                ntiles, v, d);
+    e = cudaGetLastError();
   }
-  border_kernel<<<1, 1, 0, st>>>(rel->keys, (int)rel->size, rel->tiles.blob32, rel->tiles.L32.bytes,
-                                 rel->tiles.ntiles, v, d);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof h, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(b, d, sizeof(Border), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(d);
-  *mixed = h[1] != 0;
   if (e != cudaSuccess) cudaGetLastError();
-  return e == cudaSuccess ? h[0] : -1;
+  return e == cudaSuccess;
 }
 
 // Segments of the vertices [v0, v1) over `grid` blocks; meshes numbered as in vstart.
@@ -604,16 +604,20 @@ bool mixed_cg_ready(ebb_ctx_s* ctx, ebb_rel_s* rel, const std::vector<int>& vsta
     int cut = 1;
     for (int k = 2; k < nmesh; ++k)
       if (std::abs(2LL * vstart[k] - nv) < std::abs(2LL * vstart[cut] - nv)) cut = k;
-    bool shared = false;
-    const int t = border_tile(rel, vstart[cut], &shared, ctx->stream);
-    if (t >= 0 && cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking) == cudaSuccess &&
+    // Each group maps the tiles that hold its tets.  In one order over all meshes (ids
+    // bound after finalize) both groups would map nearly every tile, so the tiles may
+    // overlap by the one at the border only; and groups that share a tet would read each
+    // other's vectors.  Otherwise one group solves them all.
+    Border border;
+    if (find_border(rel, vstart[cut], &border, ctx->stream) && !border.joined && border.last <= border.first &&
+        cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking) == cudaSuccess &&
         cudaEventCreateWithFlags(&m->fork, cudaEventDisableTiming) == cudaSuccess &&
         cudaEventCreateWithFlags(&m->join, cudaEventDisableTiming) == cudaSuccess) {
       m->ngroup = 2;
       m->group[0].v1 = m->group[1].v0 = vstart[cut];
       m->group[1].v1 = nv;
-      m->group[0].tile1 = t + (shared ? 1 : 0);
-      m->group[1].tile0 = t;
+      m->group[0].tile1 = border.last + 1;
+      m->group[1].tile0 = border.first;
       m->group[1].tile1 = rel->tiles.ntiles;
     }
   }
