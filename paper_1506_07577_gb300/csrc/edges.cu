@@ -317,13 +317,15 @@ cudaError_t launch_assemble(ebb_rel_s* rel, int model, T mu0, T lam0, const MapI
   EdgeIndex& E = rel->edges;
   const int p = sizeof(T) == 4 ? 0 : 1;
   if (E.row_off == nullptr) return cudaErrorInvalidValue;
-  bool done = false;
-  cudaError_t re = launch_row_assemble<T>(rel, model, mu0, lam0, io, st, &done);
-  // (inside a stream capture, blocks that an earlier call had to fall back to
-  // stay in use)
-  if ((re != cudaSuccess && !(re == cudaErrorStreamCaptureUnsupported && E.blocks[p] != nullptr)) || done) {
-    E.assembled[p] = re == cudaSuccess;
-    return re;
+  // K stays where it was assembled first: products that are captured (the caller's,
+  // and the CG iterations of EBB_STEP_ASSEMBLED steps) go on reading it there.
+  if (E.blocks[p] == nullptr) {
+    bool done = false;
+    const cudaError_t re = launch_row_assemble<T>(rel, model, mu0, lam0, io, st, &done);
+    if (re != cudaSuccess || done) {
+      E.assembled[p] = re == cudaSuccess;
+      return re;
+    }
   }
   if (E.blocks[p] == nullptr) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
