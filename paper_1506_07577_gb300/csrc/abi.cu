@@ -28,6 +28,7 @@ ebb_status_t set_error(ebb_ctx_s* ctx, ebb_status_t code, const std::string& msg
 
 ebb_status_t cuda_check(ebb_ctx_s* ctx, cudaError_t e, const char* what) {
   if (e == cudaSuccess) return EBB_OK;
+  cudaGetLastError();   // reported by this call: the next one's launch checks start clean
   return set_error(ctx, EBB_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
