@@ -478,7 +478,9 @@ ebb_status_t ebb_relation_vertex_order(ebb_ctx_t ctx, ebb_rel_t tets, int32_t* o
  * or is NULL.  The PCG loop runs on the device without host round trips
  * except one status read per batch of iterations.  Synchronous; fills
  * *report (may be NULL).  Errors: EBB_ERR_CG_BREAKDOWN,
- * EBB_ERR_NOT_CONVERGED (if requested), EBB_ERR_INVERTED, plus argument
+ * EBB_ERR_NOT_CONVERGED (if requested), EBB_ERR_INVERTED, EBB_ERR_CUDA while
+ * the context's stream is being captured (this and the other step calls read
+ * their results back; the capture is left as it was), plus argument
  * errors.  After a solve that ran, u and v are advanced with the last CG
  * iterate even when the call returns one of these three errors. */
 ebb_status_t ebb_cg_implicit_step(ebb_ctx_t ctx, ebb_rel_t tets, const char* u,

@@ -201,6 +201,17 @@ ebb_status_t guarded(ebb_ctx_s* ctx, F call) {
   }
 }
 
+// Steps read their results back, which a stream capture forbids.  They are refused
+// before anything is built or noted as done: work recorded in a capture does not run.
+ebb_status_t refuse_capture(ebb_ctx_s* ctx, const ebb_rel_s* tets) {
+  if (tets->verts->size == 0) return EBB_OK;   // nothing to do, nothing to wait for
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &cs);
+  if (e == cudaSuccess && cs != cudaStreamCaptureStatusNone)
+    return cuda_check(ctx, cudaErrorStreamCaptureUnsupported, "a step is synchronous");
+  return cuda_check(ctx, e, "stream state");
+}
+
 // A concrete reduction variant (AUTO resolved).
 bool valid_reduce(int r) {
   return r == EBB_REDUCE_ATOMIC || r == EBB_REDUCE_COLOR || r == EBB_REDUCE_TILED || r == EBB_REDUCE_GATHER ||
@@ -1430,6 +1441,8 @@ ebb_status_t ebb_cg_implicit_step(ebb_ctx_t ctx, ebb_rel_t tets, const char* u, 
   }
   ebb_step_params_t p = *params;
   p.reduce = reduce;
+  s = refuse_capture(ctx, tets);
+  if (s) return s;
   return guarded(ctx, [&] { return run_implicit_step(ctx, tets, (double*)pu, (double*)pv, pp, pdt, &p, report); });
 }
 
@@ -1489,6 +1502,8 @@ ebb_status_t step_vjp_entry(ebb_ctx_t ctx, ebb_rel_t tets, const char* u, const 
   }
   ebb_step_params_t p = *params;
   p.reduce = reduce;
+  s = refuse_capture(ctx, tets);
+  if (s) return s;
   return guarded(ctx, [&] {
     return run_step_vjp(ctx, tets, (const double*)pu, (const double*)pv, (const double*)pvn, pp, pdt, (double*)pgu,
                         (double*)pgv, per_tet[0], per_tet[1], &p, report);
@@ -1555,6 +1570,8 @@ ebb_status_t ebb_cg_implicit_step_batched(ebb_ctx_t ctx, ebb_rel_t tets, const c
   }
   ebb_step_params_t p = *params;
   p.reduce = reduce;
+  s = refuse_capture(ctx, tets);
+  if (s) return s;
   return guarded(
       ctx, [&] { return run_batched_step(ctx, tets, (double*)pu, (double*)pv, pp, (const int*)pb, nbatch, &p, reports); });
 }

@@ -8,6 +8,8 @@ import meshgen
 
 pytestmark = pytest.mark.gpu
 
+G = (0.0, 0.0, -9.81)
+
 
 class _Capture:
     """Capture of stream `s`, whatever the captured call does to it."""
@@ -35,6 +37,62 @@ def _mesh(n=5, **kw):
     s = torch.cuda.Stream()
     m = meshgen.cube_grid(n, jitter=0.02, seed=31)
     return m, s, DeviceTetMesh(m.X, m.tets, stream=s, **kw)
+
+
+def _params(kind, rho):
+    from paper_1506_07577_gb300 import abi
+    mu, lam = (float(x) for x in meshgen.lame_from_young(1e5, 0.4))
+    prec = abi.EBB_PREC_F64 if kind in ("f64", "vjp") else abi.EBB_PREC_F32
+    return abi.step_params(abi.EBB_STVK, 1e-3, rho, mu, lam, G, prec, rtol=1e-10)
+
+
+def _step(dm, m, kind, rho):
+    """One step (or VJP) from the same start; the two fields it updates."""
+    from paper_1506_07577_gb300 import abi
+    a = dm.vertex_field("a", torch.float64, value=meshgen.random_displacement(m.X, 5, amp=0.02, seed=3, smooth=0.01))
+    b = dm.vertex_field("b", torch.float64, value=0.05 * meshgen.random_field(m.n_verts, seed=4))
+    if kind == "vjp":
+        for k, name in enumerate(("u", "v")):
+            dm.vertex_field(name, torch.float64, value=0.01 * meshgen.random_field(m.n_verts, seed=5 + k))
+    dm.vertex_field("ids", torch.int32, ncomp=1, value=np.zeros(m.n_verts, np.int32))
+    return (a, b), {
+        "f64": lambda: abi.ebb_cg_implicit_step(dm.ctx, dm.tets, "a", "b", None, _params(kind, rho)),
+        "f32": lambda: abi.ebb_cg_implicit_step(dm.ctx, dm.tets, "a", "b", None, _params(kind, rho)),
+        "batched": lambda: abi.ebb_cg_implicit_step_batched(dm.ctx, dm.tets, "a", "b", None, "ids", 1,
+                                                            _params(kind, rho)),
+        "vjp": lambda: abi.ebb_cg_implicit_step_vjp(dm.ctx, dm.tets, "u", "v", None, "a", "b", None, None,
+                                                    _params(kind, rho)),
+    }[kind]
+
+
+@pytest.mark.parametrize("kind", ["f64", "f32", "batched", "vjp"])
+@pytest.mark.parametrize("used_before", [False, True])
+def test_refused_step_leaves_nothing_behind(kind, used_before):
+    """A step with another density, refused under capture, then called again
+    outside: as on a relation that never saw the first call.  FP64 steps repeat bit
+    for bit; FP32 ones to the rounding of their atomic sums."""
+    from paper_1506_07577_gb300 import abi
+    m, s, dm = _mesh()
+    with dm:
+        if used_before:
+            _step(dm, m, kind, 1000.0)[1]()
+        _, call = _step(dm, m, kind, 500.0)
+        with _Capture(s):
+            with pytest.raises(abi.EbbError) as ei:
+                call()
+        assert ei.value.status == abi.EBB_ERR_CUDA
+        got, call = _step(dm, m, kind, 500.0)
+        call()
+    m, s, fresh = _mesh()
+    with fresh:
+        want, call = _step(fresh, m, kind, 500.0)
+        call()
+    for x, y in zip(got, want):
+        if kind in ("f64", "vjp"):
+            tol = 0.0 if kind == "f64" else 1e-12
+        else:
+            tol = 1e-5
+        assert float((x - y).abs().max()) <= tol * float(y.abs().max())
 
 
 def test_call_after_a_refused_first_use():
