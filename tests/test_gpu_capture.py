@@ -1,5 +1,7 @@
-"""Calls under capture of the context's stream.  What a capture refuses leaves
-nothing behind that a later call would take for its own."""
+"""Calls under capture of the context's stream.  Asynchronous calls (maps, spring
+runs) are recorded and give on replay what the plain call gives; calls that read
+results back (steps) are refused, and leave nothing behind that a later call
+would take for its own."""
 import numpy as np
 import pytest
 import torch
@@ -114,3 +116,68 @@ def test_call_after_a_refused_first_use():
         assert ei.value.status == abi.EBB_ERR_CUDA
         abi.ebb_springs_run(dm.ctx, dm.tets, "q", "qd", "mass", 3.0, 1e-3, 2)
         abi.ebb_ctx_sync(dm.ctx)
+
+
+# maps that zero their outputs (a zeroing launch that the map overlaps), in the forms
+# that are launched so, and the ones that are not
+@pytest.mark.parametrize("prec,reduce", [("f64", "AUTO"), ("f64", "ATOMIC"), ("f64", "TILED"), ("f32", "TILED"),
+                                         ("f32", "COOP"), ("f32", "TILED_ORDERED"), ("f32", "GATHER")])
+def test_captured_zeroing_map_replays(prec, reduce):
+    from paper_1506_07577_gb300 import abi
+    m, s, dm = _mesh(n=9)
+    dt = torch.float64 if prec == "f64" else torch.float32
+    opts = abi.map_opts(abi.EBB_NEOHOOKEAN, 1e4, 4e4, abi.EBB_PREC_F64 if prec == "f64" else abi.EBB_PREC_F32,
+                        getattr(abi, "EBB_REDUCE_" + reduce), abi.EBB_MAP_ZERO_OUT)
+    with dm:
+        u = dm.vertex_field("u", dt, value=meshgen.random_displacement(m.X, 9, amp=0.02, seed=3, smooth=0.01))
+        w = dm.vertex_field("w", dt, value=meshgen.random_field(m.n_verts, seed=4))
+        f, kw = dm.vertex_field("f", dt), dm.vertex_field("kw", dt)
+        call = lambda: abi.ebb_map_tet_force_Kv(dm.ctx, dm.tets, "u", "w", "f", "kw", opts)
+        call()   # (first uses allocate)
+        abi.ebb_ctx_sync(dm.ctx)
+        u0, w0 = u.clone(), w.clone()
+        with _Capture(s) as g:
+            call()
+        for scale in (1.0, -0.5, 1.0):
+            u.copy_(scale * u0)
+            w.copy_(scale * w0)
+            f.fill_(7.0)
+            kw.fill_(7.0)
+            torch.cuda.synchronize()
+            g.replay()
+            g.replay()
+            torch.cuda.synchronize()
+            got = f.clone(), kw.clone()
+            call()
+            abi.ebb_ctx_sync(dm.ctx)
+            # the same sums, in the order of the atomics
+            tol = 1e-13 if prec == "f64" else 1e-5
+            for x, y in zip(got, (f, kw)):
+                assert float((x - y).abs().max()) <= tol * float(y.abs().max())
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_captured_spring_run_replays(dtype):
+    from paper_1506_07577_gb300 import abi
+    m, s, dm = _mesh(n=9, edges=True)
+    with dm:
+        dm.vertex_field("pos", dtype, value=m.X)
+        abi.ebb_springs_init(dm.ctx, dm.tets, "pos")
+        dm.vertex_field("mass", dtype, ncomp=1, value=np.linspace(0.5, 2.0, m.n_verts))
+        q, qd = dm.vertex_field("q", dtype, value=1.01 * m.X), dm.vertex_field("qd", dtype)
+        q0 = q.clone()
+        torch.cuda.synchronize()
+        run = lambda: abi.ebb_springs_run(dm.ctx, dm.tets, "q", "qd", "mass", 3.0, 1e-3, 5)
+        for _ in range(3):
+            run()
+        abi.ebb_ctx_sync(dm.ctx)
+        want = q.clone(), qd.clone()
+        with _Capture(s) as g:
+            run()
+        q.copy_(q0)
+        qd.zero_()
+        torch.cuda.synchronize()
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(q, want[0]) and torch.equal(qd, want[1])
