@@ -120,7 +120,8 @@ typedef enum { EBB_PREC_F64 = 0, EBB_PREC_F32 = 1 } ebb_precision_t;
  *           hardware atomic adds into the vertex fields.
  *   AUTO:   the autotuned choice (ebb_relation_autotune), else TILED in FP32
  *           and for the host-buffer map, and in FP64 ATOMIC, or COOP on
- *           relations of few tets (the FP64 pipe bounds FP64 maps). */
+ *           relations of few tets (the FP64 pipe bounds FP64 maps), or TILED
+ *           where thousands of tets meet in one vertex. */
 typedef enum {
   EBB_REDUCE_ATOMIC = 0,
   EBB_REDUCE_COLOR = 1,

@@ -218,23 +218,15 @@ bool valid_reduce(int r) {
          r == EBB_REDUCE_TILED_ORDERED || r == EBB_REDUCE_COOP;
 }
 
-constexpr int64_t kCoopTets = 8192;
-
-// EBB_REDUCE_AUTO: the autotuned variant for this model and precision, else by
-// precision and size.  FP32: the tiled one.  FP64 maps are bound by the FP64 pipe,
-// which the tiles' staging and reduction only add to: one thread per tet with
-// atomics from kCoopTets tets on, and below that three threads per tet, since
-// a warp's chain of FP64 instructions (64 cycles each) is then the map's time.
-// Measured, force and K w in us, tiled / atomic / three threads: StVK 2,560 tets
-// 18.5 / 16.4 / 10.3, 8,640 18.5 / 16.4 / 14.4, 40,000 41 / 37 / 40, 878,080
-// 567 / 481 / 731; neo-Hookean 8,640 20.5 / 18.5 / 18.5, 20,480 34 / 31 / 31.
+// EBB_REDUCE_AUTO: the autotuned variant for this model and precision, else the
+// tiled one in FP32 and auto_reduce_f64's in FP64.
 ebb_reduce_t resolve_reduce(const ebb_rel_s* tets, ebb_reduce_t r, int model, int precision) {
   if (r != EBB_REDUCE_AUTO) return r;
   if ((model == EBB_STVK || model == EBB_NEOHOOKEAN) && (precision == EBB_PREC_F64 || precision == EBB_PREC_F32)) {
     const int t = tets->tuned[model][precision];
     if (t >= 0) return (ebb_reduce_t)t;
   }
-  if (precision == EBB_PREC_F64) return tets->size < kCoopTets ? EBB_REDUCE_COOP : EBB_REDUCE_ATOMIC;
+  if (precision == EBB_PREC_F64) return auto_reduce_f64(tets->size, tets->vindex.most_tets);
   return EBB_REDUCE_TILED;
 }
 

@@ -137,6 +137,7 @@ struct VertexIndex {
   int* off = nullptr;
   int* ent = nullptr;
   int* order = nullptr;
+  int most_tets = 0;   // tets around one vertex, at most
 };
 
 // Edge relation with self-loops (Section 5.2) as block CSR over internal
@@ -163,6 +164,25 @@ struct EdgeIndex {
   double* epart = nullptr;
   bool springs_ready = false;
 };
+
+// EBB_REDUCE_AUTO of an untuned FP64 map, by the relation's tets and the most tets
+// around one vertex.  FP64 maps are bound by the FP64 pipe, which the tiles' staging
+// and reduction only add to: one thread per tet with atomics from kCoopTets tets on,
+// and below that three threads per tet, since a warp's chain of FP64 instructions (64
+// cycles each) is then the map's time.  Measured, force and K w in us, tiled / atomic /
+// three threads: StVK 2,560 tets 18.5 / 16.4 / 10.3, 8,640 18.5 / 16.4 / 14.4, 40,000
+// 41 / 37 / 40, 878,080 567 / 481 / 731; neo-Hookean 8,640 20.5 / 18.5 / 18.5, 20,480
+// 34 / 31 / 31.  Atomics on one vertex follow one another (2.3 ns a tet): with more
+// than kHubTets tets around a vertex the tiles' own sums are faster.  Force, tiled and
+// else, of fans of 2,500, 4,096 and 20,000 tets around one vertex: 15.0 and 14.9, 15.0
+// and 17.1, 21 and 53; diag K, neo-Hookean, of 2,500 and 3,136: 17.1 and 17.1, 17.1 and
+// 19.0.
+constexpr int64_t kCoopTets = 8192;
+constexpr int kHubTets = 2560;
+inline ebb_reduce_t auto_reduce_f64(int64_t tets, int most_tets) {
+  if (most_tets > kHubTets) return EBB_REDUCE_TILED;
+  return tets < kCoopTets ? EBB_REDUCE_COOP : EBB_REDUCE_ATOMIC;
+}
 
 struct StepScratch;   // defined in cg.cu
 

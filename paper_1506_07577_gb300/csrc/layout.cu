@@ -588,6 +588,7 @@ ebb_status_t build_layout(ebb_ctx_s* ctx, ebb_rel_s* tets, const std::vector<int
     voff[sorted[i].z + 1]++;
     voff[sorted[i].w + 1]++;
   }
+  const int most_tets = *std::max_element(voff.begin(), voff.end());   // counts still
   for (int v = 0; v < nv; ++v) voff[v + 1] += voff[v];
   {
     std::vector<int> fill(voff.begin(), voff.end() - 1);
@@ -627,6 +628,7 @@ ebb_status_t build_layout(ebb_ctx_s* ctx, ebb_rel_s* tets, const std::vector<int
     cudaGetLastError();
     return set_error(ctx, EBB_ERR_NOMEM, std::string("building the tet layout: ") + cudaGetErrorString(e));
   }
+  tets->vindex.most_tets = most_tets;
   tets->tiles.ntiles = ntiles;
   return EBB_OK;
 }
