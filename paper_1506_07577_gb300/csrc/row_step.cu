@@ -560,6 +560,15 @@ ebb_status_t ensure_row_step(ebb_ctx_s* ctx, ebb_rel_s* tets, bool* fits) {
   return EBB_OK;
 }
 
+// A solve that goes on past rounding (rtol 0) ends when r.r or r.z underflows: 1 / r.z
+// then overflows and p.Ap, which the kernel has from differences, is no number to
+// trust.  Such a solve is done, not broken down.  1e-290: diag(A) up to 1e18 lies
+// between the two; the residual has to be past rounding too.
+ebb_status_t solve_status(const RowResult& h) {
+  const bool underflow = h.iter > 0 && h.rr < 1e-290 && h.rr <= 1e-32 * h.bb;
+  return h.status == EBB_ERR_CG_BREAKDOWN && underflow ? EBB_OK : h.status;
+}
+
 struct RowVjp {
   double *gu, *gv, *gmu, *glam;
   const double* v_next;
@@ -628,7 +637,7 @@ ebb_status_t row_step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v
     e = solve<PT>(ca, pin, m.grid, st);
     if (e == cudaSuccess && vjp) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_check(ctx, e, "CG solve");
-    if (vjp && s->host->status != EBB_OK)
+    if (vjp && solve_status(*s->host) != EBB_OK)
       return set_error(ctx, s->host->status, "forward solve failed inside the step VJP");
     ca.fresh = false;   // the adjoint solve takes the same matrix
   }
@@ -652,7 +661,7 @@ ebb_status_t row_step_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_check(ctx, e, "step finish");
   const RowResult h = *s->host;
-  status = h.status;
+  status = solve_status(h);
   const double rel = h.bb > 0.0 ? std::sqrt(h.rr / h.bb) : 0.0;
   if (rep) {
     rep->iters = h.iter;
