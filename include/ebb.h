@@ -476,8 +476,12 @@ ebb_status_t ebb_relation_vertex_order(ebb_ctx_t ctx, ebb_rel_t tets, int32_t* o
  *   A dv = b by Jacobi PCG from dv = 0 (rows/cols of pinned vertices
  *   removed), v += dv, u += dt v.
  * `pinned` names a U8 or I32 one-component vertex field (nonzero = pinned),
- * or is NULL.  The PCG loop runs on the device without host round trips
- * except one status read per batch of iterations.  Synchronous; fills
+ * or is NULL.  FP64 steps assemble dt^2 K(x_n) into library-owned rows and solve on
+ * them (bitwise reproducible, whatever params->reduce names), unless a vertex has
+ * more than 128 tets, the rows' memory cannot be allocated, or params->flags asks for
+ * the edge relation; then, and in mixed precision, K p is a map in the variant
+ * params->reduce.  The PCG loop runs on the device without host round trips
+ * except, in some forms, one status read per batch of iterations.  Synchronous; fills
  * *report (may be NULL).  Errors: EBB_ERR_CG_BREAKDOWN,
  * EBB_ERR_NOT_CONVERGED (if requested), EBB_ERR_INVERTED, EBB_ERR_CUDA while
  * the context's stream is being captured (this and the other step calls read
