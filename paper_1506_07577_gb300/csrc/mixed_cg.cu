@@ -13,9 +13,8 @@
 //   A        q = M p + dt^2 acc, p.q                                      | alpha
 //   B        r -= alpha q, z = r / diag A, r.z, r.r                       | beta
 //   C        p' = z + beta p, its FP32 copy, acc = 0                      | (b)
-// with a grid barrier at each |; p and p' alternate between two arrays, so that y
-// can be late.  At (b) the walkers' first tile copies are already on their way:
-// the producers wait there themselves.  The arithmetic is the separate kernels'.
+// with a grid barrier at each |, four to an iteration; p and p' alternate between two
+// arrays, so that y can be late.  The arithmetic is the separate kernels'.
 //
 // A batch is solved as two groups of meshes by two such kernels at once, each with
 // two walkers per SM: nothing ties them together, so that one group's vectors and
@@ -191,13 +190,6 @@ __device__ __forceinline__ void segment_totals(MixedShared& sh, const double* pa
   }
 }
 
-// The producers' gate at the end of an iteration (b).
-struct IterationGate {
-  const unsigned* bar;
-  unsigned target;
-  __device__ __forceinline__ bool operator()() const { return wait_acquire(bar, target); }
-};
-
 template <typename SH, int MODEL, typename PT>
 __global__ void __launch_bounds__(SH::threads, SH::threads > 512 ? 1 : 2) mixed_cg_kernel(MixedArgs a) {
   constexpr int kWalkers = SH::walkers, kVecThreads = SH::vec, kMixThreads = SH::threads;
@@ -302,9 +294,8 @@ __global__ void __launch_bounds__(SH::threads, SH::threads > 512 ? 1 : 2) mixed_
     // everyone sees the same count: it changes only between (beta) and (b)
     if (__ldcg(a.ctl + 1) == 0u) break;
     if (maps) {
-      const IterationGate gate{bar, round * gridDim.x};
-      if (n_my > 0 && !tile_map_pass<float, MODEL, OP_KV, true, false, IterationGate>(
-                          V, n_my, it * n_my, nv, a.blobs, a.L, a.perm, a.mu0, a.lam0, io, a.err, -1, kWaitCycles, gate))
+      if (n_my > 0 && !tile_map_pass<float, MODEL, OP_KV, true, false>(V, n_my, it * n_my, nv, a.blobs, a.L, a.perm,
+                                                                       a.mu0, a.lam0, io, a.err, -1, kWaitCycles))
         sh.bad = 1;
     } else if (it > 0) {
       finish_y(pn, tid - SH::map_threads, 32 * SH::aux);
@@ -418,8 +409,6 @@ __global__ void __launch_bounds__(SH::threads, SH::threads > 512 ? 1 : 2) mixed_
     pn = t;
     ++it;
     grid_arrive(bar, round);
-    // The producers wait for (b) themselves; the rest may not read the count
-    // before it.
     ok = grid_join(sh, bar, round);
   }
   if (ok && it > 0) finish_y(pn, tid, kMixThreads);

@@ -135,8 +135,10 @@ __device__ __forceinline__ bool grid_join(RowCgShared<NP>& sh, const unsigned* b
 // Grid-wide sums of kSums values per participating thread (the first NP), and
 // a grid barrier: every block writes its partials, waits until all have, and
 // adds the partials in block order, one value per warp, so that every block
-// obtains the same sums (in sh.tot).  Two sets of partials alternate: a block
-// writes a set again only after a barrier in between.
+// obtains the same sums (in sh.tot).  A block writes its partials again only after
+// the barrier at the end of an iteration, which every block reaches with the sums
+// read; the count of rounds rises by two between sums, so they stay in one of the
+// two sets.
 template <int NP>
 __device__ __forceinline__ bool grid_sum(RowCgShared<NP>& sh, const double (&x)[kSums], double* part, unsigned* bar,
                                          unsigned& round) {

@@ -189,19 +189,11 @@ __device__ __forceinline__ void st_part4(double* p, double x, double y, double z
   reinterpret_cast<double2*>(p)[1] = make_double2(z, 0.0);
 }
 
-// `gate` is asked by the producer before its first gather, when its first blob
-// copies are on their way: it waits until the vertex fields may be read (and
-// returns false if it gave up).
-struct OpenGate {
-  __device__ __forceinline__ bool operator()() const { return true; }
-};
-
-template <typename T, int MODEL, int OPS, bool AOS, bool ORD, typename Gate = OpenGate>
+template <typename T, int MODEL, int OPS, bool AOS, bool ORD>
 __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_my, int jbase, int nv,
                                               const unsigned char* __restrict__ blobs, const BlobLayout& L,
                                               const int* __restrict__ perm, T mu0, T lam0, const MapIO<T>& io,
-                                              int* err, int drop_tile, long long wait_cycles,
-                                              const Gate& gate = Gate()) {
+                                              int* err, int drop_tile, long long wait_cycles) {
   using Z = TileSmem<T, OPS>;
   constexpr int TT = Z::TT, NF = Z::NF, RB = Z::RB, RV = Z::RV;
   unsigned char* ring = V.ring;
@@ -248,7 +240,6 @@ __device__ __forceinline__ bool tile_map_pass(const TileView<T, OPS>& V, int n_m
         const int sb = JJ % RB, sv = JJ % RV;
         bool ok = mbar_wait_or_abort(&full_b[sb], (JJ / RB) & 1u, abort_flag, wait_cycles);
         if (ok) pend &= ~(1u << sb);
-        if (jj == 0) ok = gate() && ok;
         ok = ok && (JJ < RV || mbar_wait_or_abort(&empty_v[sv], ((JJ / RV) - 1) & 1u, abort_flag, wait_cycles));
         if (__any_sync(0xffffffffu, !ok)) {
           bad = true;
