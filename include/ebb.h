@@ -334,11 +334,17 @@ ebb_status_t ebb_map_tet_force_Kv_host(ebb_ctx_t ctx, ebb_rel_t tets, const char
  * assembled before in that precision): one 3x3 block per edge and self-loop,
  * the sum over the tets that contain both vertices of the element blocks
  * K_ab[c][d] = V (dP(e_d b_b^T) b_a)_c -- the dP of ebb_map_tet_Kv applied to
- * one displacement component at one corner -- added with atomics (the block
- * sums are not bitwise reproducible).  The blocks are library-owned (9 values
- * per block in the assembly precision).  ebb_spmv_tet_K adds K w into Kw_out
- * with the K last assembled in opts->precision (8 lanes per vertex row,
- * fixed summation order); opts->model and ->reduce are not used by the
+ * one displacement component at one corner.  K is library-owned: rows of three
+ * lanes per vertex, each block the sum of its tets' records in a fixed order
+ * (bitwise reproducible); where a vertex has more than 128 tets, or the rows do
+ * not fit when K is first assembled in that precision, blocks of 9 values instead,
+ * for good, added with atomics (their sums are not bitwise reproducible).  Memory
+ * held with the relation, per value of the assembly precision: 72 per tet and
+ * about 160 per vertex of a grid for the rows, 9 per block otherwise, and 48 bytes
+ * per tet plus some 200 per vertex for the rows' pattern (from finalize with
+ * EBB_FINALIZE_EDGES, shared with FP64 steps).  ebb_spmv_tet_K adds K w into Kw_out
+ * with the K last assembled in opts->precision (fixed summation order);
+ * opts->model and ->reduce are not used by the
  * product, opts->flags may hold EBB_MAP_ZERO_OUT.  Fields as for the maps.
  * Errors: as for the maps; EBB_ERR_STATE without EBB_FINALIZE_EDGES, or for
  * a product before any assembly in that precision. */
@@ -480,7 +486,11 @@ ebb_status_t ebb_relation_vertex_order(ebb_ctx_t ctx, ebb_rel_t tets, int32_t* o
  * them (bitwise reproducible, whatever params->reduce names), unless a vertex has
  * more than 128 tets, the rows' memory cannot be allocated, or params->flags asks for
  * the edge relation; then, and in mixed precision, K p is a map in the variant
- * params->reduce.  The PCG loop runs on the device without host round trips
+ * params->reduce.  The rows are allocated by the first such step and held with the
+ * relation: 624 bytes per tet and about 1.6 KB per vertex of a grid, their pattern
+ * included (some 10 GB for 10.5 M tets).  With rtol 0 the solve goes on until the
+ * residual underflows or max_iters is reached; one whose right-hand side is below
+ * 1e-150 in norm may end in EBB_ERR_CG_BREAKDOWN.  The PCG loop runs on the device without host round trips
  * except, in some forms, one status read per batch of iterations.  Synchronous; fills
  * *report (may be NULL).  Errors: EBB_ERR_CG_BREAKDOWN,
  * EBB_ERR_NOT_CONVERGED (if requested), EBB_ERR_INVERTED, EBB_ERR_CUDA while
