@@ -323,7 +323,7 @@ __global__ void batch_finish_kernel(int n, double dt, const double* __restrict__
 // Scratch of the batched step (owned by the relation).
 struct BatchScratch {
   int nv = 0, nmesh = 0;
-  const void* batch_ptr = nullptr;
+  const void* batch_ptr = nullptr;   // the ids the tables were built from; set when all are
   int* table = nullptr;              // blk_mesh | blk_v0 | blk_v1 | mesh_blk0 | mesh_nblk
   BatchTable tb{};
   void* acc[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -411,7 +411,6 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   tets->batch = s;
   s->nv = nv;
   s->nmesh = nmesh;
-  s->batch_ptr = batch;
   s->vstart = vstart;
   const size_t n = (size_t)3 * nv;
   e = cudaMalloc(&s->table, sizeof(int) * (3 * (size_t)nb + 2 * (size_t)nmesh));
@@ -455,6 +454,8 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   s->tb.mesh_blk0 = s->table + 3 * nb;
   s->tb.mesh_nblk = s->table + 3 * nb + nmesh;
   s->h_sc.resize(nmesh);
+  s->h_res.resize(nmesh);
+  s->batch_ptr = batch;   // last: a call that host memory failed leaves no finished scratch
   return EBB_OK;
 }
 
@@ -602,7 +603,6 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
   }
   batch_finish_kernel<<<4 * 152, 256, 0, st>>>(n, prm->dt, s->y, u, v);
   e = cudaGetLastError();
-  s->h_res.resize(nmesh);
   if (e == cudaSuccess)
     e = one_launch ? cudaMemcpyAsync(s->h_res.data(), mixed_results(s->mixed), (size_t)nmesh * sizeof(MixedResult),
                                      cudaMemcpyDeviceToHost, st)

@@ -49,7 +49,18 @@ inline cudaError_t fake_capturing(cudaStream_t, cudaStreamCaptureStatus* s) {
   return cudaSuccess;
 }
 
+inline cudaError_t fake_stream(cudaStream_t* s, unsigned) {
+  *s = nullptr;
+  return cudaSuccess;
+}
+inline cudaError_t fake_event(cudaEvent_t* e, unsigned) {
+  *e = nullptr;
+  return cudaSuccess;
+}
+
 #define cudaMalloc fake_malloc
+#define cudaStreamCreateWithFlags fake_stream
+#define cudaEventCreateWithFlags fake_event
 #define cudaFree fake_free
 #define cudaMemcpyAsync fake_memcpy
 #define cudaMemsetAsync fake_memset

@@ -36,3 +36,11 @@ def test_assembled_stiffness_stays_in_its_storage(tmp_path):
     got = _run(tmp_path, "assembly_storage", ["edges.cu", "row_matrix.cu"])
     assert got == [(0, 0, 1), (0, 0, 1), (0, 0, 1),   # FP32: no room, room again, captured
                    (1, 0, 0), (0, 1, 0), (0, 1, 0)]   # FP64: first use captured, not captured, captured
+
+
+def test_batch_scratch_after_host_memory_ran_out(tmp_path):
+    """(first call failed, second call's tables whole), the first call's k-th host
+    allocation failing: a half-built scratch is not taken for a finished one."""
+    got = _run(tmp_path, "batch_scratch", [])
+    assert len(got) > 5 and got[-1] == (0, 1)
+    assert all(g == (1, 1) for g in got[:-1]), got
