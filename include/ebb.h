@@ -544,7 +544,8 @@ ebb_status_t ebb_cg_implicit_step_vjp_at(ebb_ctx_t ctx, ebb_rel_t tets, const ch
  * meshes of uneven sizes; the per-mesh step is exactly the one above).
  * `batch` names an I32 one-component vertex field giving each vertex its mesh
  * id in [0, nbatch); ids must be non-decreasing along verts (each mesh's
- * vertices contiguous) and every id must occur.  Bind the field as
+ * vertices contiguous) and every id must occur.  The ids are read by the first
+ * step after the field is bound: bind it again after changing them in place.  Bind the field as
  * "batch" before ebb_relation_finalize so tets are ordered mesh by mesh and
  * a tet joining two meshes is rejected (EBB_ERR_KEY); with ids bound later,
  * or others than those, the results are the same and the tets' order costs

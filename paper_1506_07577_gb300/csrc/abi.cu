@@ -514,6 +514,7 @@ ebb_status_t ebb_field_bind(ebb_rel_t rel, const char* name, ebb_dtype_t dtype, 
   f.ncomp = ncomp;
   f.ptr = device_ptr;
   f.key_target = key_target;
+  f.bind = ++ctx->binds;
   rel->fields[name] = f;
   return EBB_OK;
 }
@@ -1564,8 +1565,10 @@ ebb_status_t ebb_cg_implicit_step_batched(ebb_ctx_t ctx, ebb_rel_t tets, const c
   p.reduce = reduce;
   s = refuse_capture(ctx, tets);
   if (s) return s;
-  return guarded(
-      ctx, [&] { return run_batched_step(ctx, tets, (double*)pu, (double*)pv, pp, (const int*)pb, nbatch, &p, reports); });
+  const uint64_t bind = find_field(tets->verts, batch)->bind;
+  return guarded(ctx, [&] {
+    return run_batched_step(ctx, tets, (double*)pu, (double*)pv, pp, (const int*)pb, bind, nbatch, &p, reports);
+  });
 }
 
 }  // extern "C"

@@ -323,7 +323,8 @@ __global__ void batch_finish_kernel(int n, double dt, const double* __restrict__
 // Scratch of the batched step (owned by the relation).
 struct BatchScratch {
   int nv = 0, nmesh = 0;
-  const void* batch_ptr = nullptr;   // the ids the tables were built from; set when all are
+  int* ids = nullptr;                // the ids the tables were built from
+  uint64_t bind = 0;                 // and the binding they came from; set when all tables are
   int* table = nullptr;              // blk_mesh | blk_v0 | blk_v1 | mesh_blk0 | mesh_nblk
   BatchTable tb{};
   void* acc[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -361,6 +362,7 @@ void free_batch_scratch(ebb_rel_s* rel) {
   cudaFree(s->sc);
   cudaFree(s->n_active);
   cudaFree(s->p2);
+  cudaFree(s->ids);
   free_mixed_plan(s->mixed);
   if (s->chunk) cudaGraphExecDestroy(s->chunk);
   if (s->ev) cudaEventDestroy(s->ev);
@@ -371,12 +373,40 @@ void free_batch_scratch(ebb_rel_s* rel) {
 
 namespace {
 
+__global__ void ids_differ_kernel(int n, const int* __restrict__ a, const int* __restrict__ b, int* differ) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    if (a[i] != b[i]) *differ = 1;
+}
+
+// Are these the ids that the tables were built from?
+ebb_status_t same_ids(ebb_ctx_s* ctx, BatchScratch* s, const int* batch, bool* same) {
+  int differ = 1;
+  cudaError_t e = cudaMemsetAsync(s->n_active, 0, sizeof(int), ctx->stream);
+  if (e == cudaSuccess) {
+    ids_differ_kernel<<<std::min((s->nv + 255) / 256, 4 * 152), 256, 0, ctx->stream>>>(s->nv, batch, s->ids,
+                                                                                     s->n_active);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&differ, s->n_active, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  *same = differ == 0;
+  return cuda_check(ctx, e, "comparing batch ids");
+}
+
 // Validate the batch field (ids non-decreasing from 0, each mesh non-empty)
-// and build the block table.
-ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, int nmesh) {
+// and build the block table, once per binding of the field whose ids are others.
+ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, uint64_t bind, int nmesh) {
   const int nv = (int)tets->verts->size;
   BatchScratch* s = tets->batch;
-  if (s && s->nv == nv && s->nmesh == nmesh && s->batch_ptr == batch) return EBB_OK;
+  if (s && s->bind != 0 && s->nv == nv && s->nmesh == nmesh) {
+    bool same = s->bind == bind;
+    if (!same) {   // bound again: the same memory may hold other ids
+      const ebb_status_t cs = same_ids(ctx, s, batch, &same);
+      if (cs) return cs;
+      if (same) s->bind = bind;
+    }
+    if (same) return EBB_OK;
+  }
   free_batch_scratch(tets);
   std::vector<int> hb(nv);
   cudaError_t e = cudaMemcpyAsync(hb.data(), batch, sizeof(int) * nv, cudaMemcpyDeviceToHost, ctx->stream);
@@ -426,6 +456,7 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   if (e == cudaSuccess) e = cudaMalloc(&s->part, 2 * (size_t)nb * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&s->sc, (size_t)nmesh * sizeof(MeshCg));
   if (e == cudaSuccess) e = cudaMalloc(&s->n_active, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&s->ids, (size_t)nv * sizeof(int));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -442,6 +473,7 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   // on the solve's stream: a copy from pageable memory may return before it has
   // landed, and this stream does not wait for the legacy default one
   e = cudaMemcpyAsync(s->table, host.data(), sizeof(int) * host.size(), cudaMemcpyHostToDevice, s->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(s->ids, hb.data(), sizeof(int) * nv, cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) {
     free_batch_scratch(tets);
@@ -455,7 +487,7 @@ ebb_status_t prepare_batch(ebb_ctx_s* ctx, ebb_rel_s* tets, const int* batch, in
   s->tb.mesh_nblk = s->table + 3 * nb + nmesh;
   s->h_sc.resize(nmesh);
   s->h_res.resize(nmesh);
-  s->batch_ptr = batch;   // last: a call that host memory failed leaves no finished scratch
+  s->bind = bind;   // last: a call that host memory failed leaves no finished scratch
   return EBB_OK;
 }
 
@@ -647,10 +679,11 @@ ebb_status_t batch_impl(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, c
 }  // namespace
 
 ebb_status_t run_batched_step(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, const void* pinned,
-                              const int* batch, int nmesh, const ebb_step_params_t* p, ebb_cg_report_t* reps) {
+                              const int* batch, uint64_t bind, int nmesh, const ebb_step_params_t* p,
+                              ebb_cg_report_t* reps) {
   if (cudaSetDevice(ctx->device) != cudaSuccess) return set_error(ctx, EBB_ERR_CUDA, "cudaSetDevice failed");
   if (tets->vindex.off == nullptr) return set_error(ctx, EBB_ERR_STATE, "relation has no vertex index");
-  ebb_status_t s = prepare_batch(ctx, tets, batch, nmesh);
+  ebb_status_t s = prepare_batch(ctx, tets, batch, bind, nmesh);
   if (s) return s;
   return p->precision == EBB_PREC_F64
              ? batch_impl<double>(ctx, tets, u, v, (const unsigned char*)pinned, p, nmesh, reps)

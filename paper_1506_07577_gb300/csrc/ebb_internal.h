@@ -23,6 +23,7 @@ struct Field {
   int ncomp = 1;
   void* ptr = nullptr;
   ebb_rel_s* key_target = nullptr;
+  uint64_t bind = 0;   // count of the context's field bindings at this one
 };
 
 // Per-tet streams in the layout the kernels read.  Matrices are 9 planes of
@@ -230,6 +231,7 @@ struct ebb_ctx_s {
   std::string last_error;
   int* d_err = nullptr;     // device status word (ERRW_WORDS ints)
   int* h_err = nullptr;     // pinned host mirror
+  uint64_t binds = 0;       // field bindings so far
   std::vector<ebb_rel_s*> rels;
 };
 
@@ -399,9 +401,10 @@ cudaError_t launch_adjoint_map(ebb_rel_s* rel, double mu0, double lam0, const do
                                const double* w, double* acc_kl, double* acc_xq, double* gmu, double* glam, double dt,
                                cudaStream_t st);
 
-// Batched implicit step (batched.cu).
+// Batched implicit step (batched.cu).  `bind`: the ids field's Field::bind.
 ebb_status_t run_batched_step(ebb_ctx_s* ctx, ebb_rel_s* tets, double* u, double* v, const void* pinned,
-                              const int* batch, int nmesh, const ebb_step_params_t* p, ebb_cg_report_t* reps);
+                              const int* batch, uint64_t bind, int nmesh, const ebb_step_params_t* p,
+                              ebb_cg_report_t* reps);
 void free_batch_scratch(ebb_rel_s* rel);
 
 // Staging in the vertex-interleaved layout (reorder.cu): da/db[4 i + c] =

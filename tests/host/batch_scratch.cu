@@ -56,12 +56,12 @@ int main() {
     bool failed = false;
     allocs_left = k;
     try {
-      failed = ebb::prepare_batch(&ctx, &tets, ids, 3) != EBB_OK;
+      failed = ebb::prepare_batch(&ctx, &tets, ids, 1, 3) != EBB_OK;
     } catch (const std::bad_alloc&) {
       failed = true;
     }
     allocs_left = -1;
-    bool whole = ebb::prepare_batch(&ctx, &tets, ids, 3) == EBB_OK;
+    bool whole = ebb::prepare_batch(&ctx, &tets, ids, 1, 3) == EBB_OK;
     const ebb::BatchScratch* s = tets.batch;
     whole = whole && s && s->tb.nblocks == 3 && s->tb.blk_mesh && s->tb.mesh_nblk && s->h_sc.size() == 3 &&
             s->vstart.size() == 4;

@@ -51,3 +51,36 @@ def test_each_call_uses_its_parameters(prec, reduce):
                 want = _step(dm, b, prec, model, reduce, **c)
             for x, y in zip(g, want):
                 assert float((x - y).abs().max()) <= tol * float(y.abs().max()), (model, c)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_ids_changed_in_place_and_bound_again(prec):
+    """Three grids as two meshes, first the first two together, then the last two, in
+    the same memory.  Three CG iterations: their scalars are the meshes' own."""
+    from paper_1506_07577_gb300 import abi
+    b = meshgen.cube_grid_batch(np.array([4, 3, 4]), jitter=0.02, seed=202)
+    splits = [np.array(s, np.int32)[b.batch] for s in ((0, 0, 1), (0, 1, 1))]
+    prm = abi.step_params(abi.EBB_STVK, 5e-3, 1000.0, 3e4, 5e4, G,
+                          abi.EBB_PREC_F64 if prec == "f64" else abi.EBB_PREC_F32, max_iters=3, rtol=1e-12)
+
+    def run(dm, ids):
+        dm._tensors["ids"].copy_(torch.from_numpy(ids))
+        dm._tensors["u"].zero_()
+        dm._tensors["v"].copy_(torch.from_numpy(0.05 * meshgen.random_field(b.X.shape[0], seed=13).T))
+        torch.cuda.synchronize()
+        dm.bind("ids", dm._tensors["ids"])
+        abi.ebb_cg_implicit_step_batched(dm.ctx, dm.tets, "u", "v", "pinned", "ids", 2, prm)
+        return dm._tensors["v"].clone()
+
+    with _mesh(b) as dm:
+        dm.vertex_field("ids", torch.int32, ncomp=1)
+        got = [run(dm, splits[k]) for k in (0, 1, 0, 0)]
+    want = []
+    for k in (0, 1):
+        with _mesh(b) as dm:
+            dm.vertex_field("ids", torch.int32, ncomp=1)
+            want.append(run(dm, splits[k]))
+    tol = 1e-9 if prec == "f64" else 1e-5
+    for g, k in zip(got, (0, 1, 0, 0)):
+        assert float((g - want[k]).abs().max()) <= tol * float(want[k].abs().max())
+    assert float((want[0] - want[1]).abs().max()) > 10 * tol * float(want[0].abs().max())
