@@ -448,8 +448,9 @@ element_block_kernel(int nt, int nv, const int4* __restrict__ keys, const int* _
   if constexpr (STAGE) {
     __syncwarp();
     const int w0 = (int)threadIdx.x & ~31, lane = threadIdx.x & 31;
-    const int n = min(32, nt - (blockIdx.x * kElemThreads + w0)) * L;   // words of the warp's records
-    T* dst = elem + (size_t)(blockIdx.x * kElemThreads + w0) * L;
+    const int t0 = (int)blockIdx.x * kElemThreads + w0;
+    const int n = warp_tets(t0, nt) * L;   // words of the warp's records
+    T* dst = elem + (size_t)t0 * L;
     for (int x = lane; x < n; x += 32) dst[x] = s_rec[w0 + x / L][x % L];
   }
 }

@@ -67,6 +67,13 @@ struct RowView {
   const int* __restrict__ col;
 };
 
+// Tets of a warp that starts at tet t0 (signed: a block's second warp may start
+// past the last tet).
+__host__ __device__ inline int warp_tets(int t0, int nt) {
+  const int n = nt - t0;
+  return n < 0 ? 0 : (n < 32 ? n : 32);
+}
+
 // First slice of block b of `grid`, which take consecutive slices.
 __host__ __device__ inline int first_slice(int b, int grid, int nslice) {
   return (int)((long long)b * nslice / grid);
